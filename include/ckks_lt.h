@@ -107,9 +107,9 @@ ckks_status ckks_ctx_destroy(ckks_ctx* ctx);
  * equal beta_max*2*(L+k)*N.  The same key serves every algorithm and split:
  * the hoisted form swk~_r = phi_{-r}(swk_r) of Algorithms 1-2 is applied as
  * an index gather on the digits.  r is taken mod N/2; replacing a key is
- * allowed when no queued work uses it.  The library stores the key with its
- * two components interleaved per word ([beta_max][L+k][N] pairs), so that
- * every kernel reads one 16-byte word per digit word; the upload converts. */
+ * allowed when no queued work uses it.  The upload converts the key to the
+ * library's own layout, at 5 bytes a word for moduli between 2^32 and 2^40
+ * and 8 bytes otherwise; words at or above their modulus are reduced. */
 ckks_status ckks_upload_rotation_key(ckks_ctx* ctx, int32_t r, const uint64_t* host, size_t n_words);
 /* Same, from a device buffer the library reads in stream order on `stream`
  * (the conversion is a kernel there; `dev` must stay valid until it ran). */
@@ -134,7 +134,9 @@ int ckks_has_rotation_key(const ckks_ctx* ctx, int32_t r);
  * a factored DFT (CoeffToSlot / SlotToCoeff). */
 ckks_status ckks_upload_diagonals(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, int32_t offset0,
                                   int32_t stride, uint32_t level, const uint64_t* host, size_t n_words);
-/* Same, from a device buffer the library copies (stream-ordered on `stream`). */
+/* Same, from a device buffer the library reads in stream order on `stream`
+ * (the conversion to the library's layout, as for the keys, is a kernel there;
+ * `dev` must stay valid until it ran). */
 ckks_status ckks_upload_diagonals_device(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, int32_t offset0,
                                          int32_t stride, uint32_t level, const uint64_t* dev, size_t n_words,
                                          void* stream);
@@ -143,8 +145,8 @@ ckks_status ckks_upload_diagonals_device(ckks_ctx* ctx, ckks_diags** out, uint32
  * to stage twice in device memory. */
 ckks_status ckks_diags_create(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, int32_t offset0, int32_t stride,
                               uint32_t level);
-/* Copy diagonals [first, first + count) from a device buffer
- * [count][level + k][N] (stream-ordered). */
+/* Write diagonals [first, first + count) from a device buffer
+ * [count][level + k][N] (converted by a kernel in stream order). */
 ckks_status ckks_diags_write_device(ckks_diags* f, uint32_t first, uint32_t count, const uint64_t* dev,
                                    size_t n_words, void* stream);
 ckks_status ckks_free_diags(ckks_diags* f);
@@ -280,13 +282,12 @@ ckks_status lt_autotune_batch(ckks_ctx* ctx, lt_algo algo, uint32_t count, const
 
 /* The tile lt_autotune measured for the shape (algo, f, level) besides its
  * split: outer rotation indices per CTA of the diagonal multiply-accumulate
- * kernel (Alg. 2 lines 8-14) and positions per CTA, each 0 for the default
- * (outer: the next power of two >= n'3, at most 8; positions: 128, four
- * CTAs per SM, or two with 8 outer indices).  lt_autotune times the default,
- * half the outer indices, and 256 positions for its chosen split, and
- * lt_eval uses the fastest whenever it runs that split for that shape;
- * results do not depend on the tile.  Returns 1 and writes the tile, 0 if
- * the shape was not tuned, -1 on a null argument. */
+ * kernel (Alg. 2 lines 8-14), 0 for the default, the next power of two
+ * >= n'3, at most 8.  lt_autotune times the default and half of it for its
+ * chosen split, and lt_eval uses the faster whenever it runs that split for
+ * that shape; results do not depend on the tile.  positions_per_cta is always
+ * written as 0: the kernel has one size, 128 positions per CTA.  Returns 1 and
+ * writes the tile, 0 if the shape was not tuned, -1 on a null argument. */
 int32_t lt_tuned_tile(const ckks_ctx* ctx, lt_algo algo, const ckks_diags* f, uint32_t level, uint32_t* outer_per_cta,
                       uint32_t* positions_per_cta);
 
@@ -397,11 +398,12 @@ ckks_status ckks_selftest_bounded_wait(ckks_ctx* ctx, uint32_t limit_ms, void* s
 ckks_status ckks_debug_diag_mac_waits(ckks_ctx* ctx, uint64_t wait_limit_ns, uint32_t starve_step);
 
 /* Test hook: every later LT on the context runs the diagonal kernel with this
- * tile (see lt_tuned_tile; outer_per_cta 0 or a power of two up to 8, at
- * most the default; positions_per_cta 0, 128, 256 or 512), instead of the tuned or
- * default one; (0, 0) restores the normal choice.  Results do not depend on
- * the tile, which is what the test checks.  It changes the context like an
- * upload (no evaluation call may overlap it). */
+ * many outer indices per CTA (see lt_tuned_tile; 0 or a power of two up to 8,
+ * at most the default), instead of the tuned or default number; 0 restores
+ * the normal choice.  positions_per_cta is 0, 128, 256 or 512 and has no
+ * effect (128 positions per CTA).  Results do not depend on the tile, which is
+ * what the test checks.  It changes the context like an upload (no evaluation
+ * call may overlap it). */
 ckks_status ckks_debug_diag_mac_tile(ckks_ctx* ctx, uint32_t outer_per_cta, uint32_t positions_per_cta);
 
 const char* ckks_last_error(void);

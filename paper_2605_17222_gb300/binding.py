@@ -348,8 +348,8 @@ class Context:
         return [buf[i].tuple() for i in range(n)]
 
     def tuned_tile(self, algo: str, diags: "Diagonals", level: int):
-        """(outer indices per CTA, positions per CTA) lt_autotune measured for the
-        shape (0 = default), or None if the shape was not tuned (lt_tuned_tile)."""
+        """(outer indices per CTA, 0) lt_autotune measured for the shape (0 = default;
+        the second value is unused, see lt_tuned_tile), or None if the shape was not tuned (lt_tuned_tile)."""
         k3, run = ctypes.c_uint32(), ctypes.c_uint32()
         r = lib().lt_tuned_tile(self.h, ALGOS[algo], diags.handle, level, ctypes.byref(k3), ctypes.byref(run))
         if r < 0:

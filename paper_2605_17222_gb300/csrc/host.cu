@@ -97,7 +97,10 @@ bool is_prime_h(u64 n) {
 
 ModC modc_h(u64 q) {
     u128 mu = (~(u128)0) / q;  // = floor(2^128 / q) since q does not divide 2^128
-    return ModC{q, (u64)(mu >> 64), (u64)mu};
+    u32 bits = 0;
+    while (bits < 64 && (q >> bits)) bits++;
+    const u64 mu_s = (u64)(mu >> (65 - bits));  // floor(floor(2^128 / q) / 2^(65 - bits)) = floor(2^(63 + bits) / q)
+    return ModC{q, (u64)(mu >> 64), (u64)mu, mu_s, 0, 0, bits, 0};
 }
 
 u32 brv_h(u32 x, u32 bits) {
@@ -135,22 +138,25 @@ struct ckks_ctx {
     u32 log_n = 0, N = 0, L = 0, K = 0, dnum = 0, alpha = 0, beta_max = 0;
     std::vector<u64> mods;  // q_0..q_{L-1}, p_0..p_{K-1}
     DevBuf d_mods, d_psi, d_ipsi, d_lift, d_lift_sh, d_err;
+    std::vector<u64> q_bytes{0};  // bytes of the first t Q limbs of a diagonal, t <= L
+    u64 p_bytes = 0, key_bytes = 0;  // bytes of its P limbs; of a key
     std::vector<u64> lift_c, lift_sh;  // host copies: [P]_{q_t} and its Shoup companion per Q limb
     NttTables T{};
     std::map<u32, LevelConsts> levels;
-    std::map<u32, u64*> keys;  // rotation (mod N/2) -> [beta_max][L+K][N] word pairs (components interleaved)
+    std::map<u32, unsigned char*> keys;  // rotation (mod N/2) -> key (layout in kernels.h)
     std::map<std::tuple<int, u32, u32, int32_t, int32_t>, lt_split> tuned;  // (algo, level, D, stride, offset0 mod N/2)
     // DH-BSGS schedule per (level, D, stride, offset0 mod N/2, n1, n2) measured by lt_autotune:
     // true = the baby steps fused into the diagonal kernel's middle layer, TH(1, n1, n2)
     std::map<std::tuple<u32, u32, int32_t, int32_t, u32, u32>, bool> dh_fused;
-    // the diagonal kernel's tile measured by lt_autotune for a shape's tuned split (same key as `tuned`)
-    std::map<std::tuple<int, u32, u32, int32_t, int32_t>, std::pair<u32, u32>> tuned_tile;
+    // the diagonal kernel's tile (outer indices per CTA) measured by lt_autotune for a shape's tuned split
+    // (same key as `tuned`)
+    std::map<std::tuple<int, u32, u32, int32_t, int32_t>, u32> tuned_tile;
     mutable std::mutex mu;
     size_t bytes = 0;
     // failure-detection test hook of the staged diagonal kernel (ckks_debug_diag_mac_waits)
     u64 dbg_wait_ns = 0;
     u32 dbg_starve_step = ~0u;
-    u32 dbg_tile_k3 = 0, dbg_tile_run = 0;  // forced diagonal-kernel tile (ckks_debug_diag_mac_tile)
+    u32 dbg_tile_k3 = 0;  // forced diagonal-kernel tile (ckks_debug_diag_mac_tile)
     // fork/join lanes of lt_eval_batch: independent groups run on the caller's
     // stream and up to FORK_LANES - 1 more, so that one group's NTT-bound
     // phases overlap another's HBM-bound diagonal multiply-accumulate
@@ -167,6 +173,7 @@ struct ckks_ctx {
     u32 beta(u32 level) const { return (level + alpha - 1) / alpha; }
     u32 slots() const { return N / 2; }
     size_t key_words() const { return (size_t)beta_max * 2 * (L + K) * N; }
+    u64 diag_bytes(u32 level) const { return q_bytes[level] + p_bytes; }
     u32 gmod(u32 level, u32 t) const { return t < level ? t : L + (t - level); }
     u32 galois(int64_t r) const {
         int64_t rr = r % (int64_t)slots();
@@ -215,7 +222,7 @@ struct ckks_diags {
     ckks_ctx* ctx;
     u32 n_diag, level;
     int32_t offset0, stride;
-    u64* d;
+    unsigned char* d;  // [n_diag] of ctx->diag_bytes(level) bytes (layout in kernels.h)
 };
 
 // Constants that depend on the level (digit boundaries, sources of the
@@ -355,13 +362,17 @@ void release_lanes(ckks_ctx* C, cudaStream_t st) {
 // (gathered through x -> x^gal if gal) -> digits_i [beta][level+K][N].
 // Y: scratch [count][level][N].  One launch pair per transform direction
 // covers every polynomial, so small steps still fill the GPU.
+// slots: 0 for plain digits, else the slots of grouped digits (DigLayout), of
+// which the digits take the first beta.
 // extra: further elementwise jobs (FWD_COPY) to run in the forward launch.
 void op_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& cs, u32 gal,
-                        const std::vector<u64*>& digits, u64* Y, cudaStream_t st,
+                        const std::vector<u64*>& digits, u32 slots, u64* Y, cudaStream_t st,
                         const std::vector<FwdJob>* extra = nullptr) {
     const LevelConsts& LC = C->lc(level);
     const u32 N = C->N, ext = level + C->K, beta = C->beta(level);
     const u32 cnt = (u32)cs.size();
+    const DigLayout dl = slots ? grouped_digits(slots, C->log_n) : plain_digits(ext, C->log_n);
+    const u32 step = slots << FWD_STEP;
     std::vector<InvJob> ij;
     ij.reserve((size_t)cnt * level);
     for (u32 p = 0; p < cnt; p++) {
@@ -381,9 +392,9 @@ void op_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& c
             for (u32 j = first; j < first + n; j++) small = small && C->mods[j] < (1ull << 41);
             for (u32 t = 0; t < ext; t++) {
                 if (t >= first && t < first + n) continue;
-                fj.push_back(FwdJob{Yp + (size_t)first * N, digits[p] + ((size_t)b * ext + t) * N,
+                fj.push_back(FwdJob{Yp + (size_t)first * N, digits[p] + b * dl.dig + t * dl.limb,
                                     LC.dec_tab + ((size_t)b * ext + t) * C->alpha, nullptr, nullptr, 0, 0,
-                                    C->gmod(level, t), n | (small ? 1u << 16 : 0u)});
+                                    C->gmod(level, t), n | (small ? 1u << 16 : 0u) | step});
             }
         }
         // each digit's own limbs are the (gathered) input limbs: copy jobs in the same launch, after
@@ -391,17 +402,24 @@ void op_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& c
         for (u32 b = 0; b < beta; b++) {
             const u32 first = b * C->alpha, n = std::min(C->alpha, level - first);
             for (u32 j = first; j < first + n; j++)
-                fj.push_back(FwdJob{cs[p] + (size_t)j * N, digits[p] + ((size_t)b * ext + j) * N, nullptr, nullptr,
-                                    nullptr, gal, 0, j, FWD_COPY});
+                fj.push_back(FwdJob{cs[p] + (size_t)j * N, digits[p] + b * dl.dig + j * dl.limb, nullptr, nullptr,
+                                    nullptr, gal, 0, j, FWD_COPY | step});
         }
     }
     if (extra) fj.insert(fj.end(), extra->begin(), extra->end());
     launch_fwd_ntt(C->T, fj.data(), (int)fj.size(), st);
 }
 
-void op_decompose(ckks_ctx* C, u32 level, const u64* c, u32 gal, u64* digits, u64* Y, cudaStream_t st,
-                  const std::vector<FwdJob>* extra = nullptr) {
-    op_decompose_batch(C, level, std::vector<const u64*>{c}, gal, std::vector<u64*>{digits}, Y, st, extra);
+void op_decompose(ckks_ctx* C, u32 level, const u64* c, u32 gal, u64* digits, u64* Y, cudaStream_t st) {
+    op_decompose_batch(C, level, std::vector<const u64*>{c}, gal, std::vector<u64*>{digits}, 0, Y, st);
+}
+
+// P c0 (Alg. 2 line 2) as scaling jobs: the Q limbs of a plain c0 to dst, whose
+// limbs lie `limb` words apart and their blocks `slots` blocks apart.
+void lift_jobs(const ckks_ctx* C, u32 level, const u64* c0, u64* dst, u64 limb, u32 slots, std::vector<FwdJob>& out) {
+    for (u32 t = 0; t < level; t++)
+        out.push_back(FwdJob{c0 + (size_t)t * C->N, dst + t * limb, nullptr, nullptr, nullptr, C->lift_c[t],
+                             C->lift_sh[t], t, FWD_COPY | FWD_SCALE | slots << FWD_STEP});
 }
 
 // Modulus switch down of `count` polynomials over a contiguous source run:
@@ -464,33 +482,50 @@ void op_rescale(ckks_ctx* C, u32 level, const u64* x, u64* out, u64* Y, cudaStre
     op_rescale_batch(C, level, std::vector<const u64*>{x}, std::vector<u64*>{out}, Y, st);
 }
 
-const u64* key_of(ckks_ctx* C, int64_t r) {
+const unsigned char* key_of(ckks_ctx* C, int64_t r) {
     auto it = C->keys.find(C->rotkey(r));
     if (it == C->keys.end()) fail(CKKS_ENOKEY, "missing rotation key for r = " + std::to_string(C->rotkey(r)));
     return it->second;
 }
 
-void op_ks_inner(ckks_ctx* C, u32 level, const u64* digits, const u64* key, u32 gal, const u64* x0, int x0_mode,
-                 u64* out0, u64* out1, int acc, cudaStream_t st) {
-    KsArgs a{};
-    a.digits = digits;
-    a.key = key;
-    a.x0 = x0;
-    a.out0 = out0;
-    a.out1 = out1;
+// slots: 0 for plain digits, else grouped ones (DigLayout); o_slots: the same
+// for out0's blocks.
+KsArgs ks_base(const ckks_ctx* C, u32 level, u32 slots, u32 o_slots) {
+    KsArgs a;
+    memset(&a, 0, sizeof(a));
     a.mods = (const ModC*)C->d_mods.p;
     a.lift_c = C->d_lift.p;
     a.lift_sh = C->d_lift_sh.p;
+    a.err = (u32*)C->d_err.p;
+    a.dl = slots ? grouped_digits(slots, C->log_n) : plain_digits(level + C->K, C->log_n);
+    a.o_limb = (u64)std::max(1u, o_slots) * C->N;
+    a.o_blk = std::max(1u, o_slots) * BLK;
     a.level = level;
     a.ext = level + C->K;
     a.L = C->L;
     a.beta = C->beta(level);
     a.beta_max = C->beta_max;
-    a.gal = gal;
+    a.log_n = C->log_n;
+    return a;
+}
+
+void op_ks_inner(ckks_ctx* C, u32 level, const u64* digits, const unsigned char* key, u32 gal, const u64* x0, int x0_mode,
+                 u64* out0, u64* out1, int acc, cudaStream_t st) {
+    KsArgs a = ks_base(C, level, 0, 0);
+    a.e[0] = KsItem{digits, key, x0, out0, out1, gal, 0};
+    a.count = 1;
     a.x0_mode = x0 ? x0_mode : 0;
     a.accumulate = acc;
-    a.log_n = C->log_n;
-    launch_ks_inner(a, st);
+    launch_ks(a, st);
+}
+
+// The products of a list, KS_MAX at a time (see KsArgs).
+void op_ks_list(KsArgs& a, const std::vector<KsItem>& items, cudaStream_t st) {
+    for (size_t e0 = 0; e0 < items.size(); e0 += KS_MAX) {
+        a.count = (u32)std::min<size_t>(KS_MAX, items.size() - e0);
+        std::copy(items.begin() + e0, items.begin() + e0 + a.count, a.e);
+        launch_ks(a, st);
+    }
 }
 
 void op_add_gather(ckks_ctx* C, u32 nlimbs, u32 level, const u64* a, const u64* b, u64* out, u32 gal, int acc,
@@ -502,27 +537,27 @@ void op_add_gather(ckks_ctx* C, u32 nlimbs, u32 level, const u64* a, const u64* 
     launch_add_gather((const ModC*)C->d_mods.p, j.data(), (int)nlimbs, gal, acc, C->log_n, st);
 }
 
-// Tile of the diagonal kernel (0 = default; see DiagMacArgs).
-struct K6Tile {
-    u32 k3 = 0, run = 0;
-};
-
-DiagMacArgs dm_base(ckks_ctx* C, u32 level, bool with_p, const ckks_diags* f, K6Tile tile = K6Tile{}) {
+// tile: the diagonal kernel's outer indices per CTA (0 = default; see DiagMacArgs).
+DiagMacArgs dm_base(ckks_ctx* C, u32 level, bool with_p, const ckks_diags* f, u32 tile = 0) {
     DiagMacArgs a;
     memset(&a, 0, sizeof(a));
-    a.tile_k3 = tile.k3;
-    a.tile_run = tile.run;
+    a.tile_k3 = tile;
     a.mods = (const ModC*)C->d_mods.p;
     a.lift_c = C->d_lift.p;
     a.lift_sh = C->d_lift_sh.p;
     a.diags = f->d;
+    a.diag_stride = C->diag_bytes(f->level);
+    a.diag_p = C->q_bytes[f->level];
     a.level = level;
     a.ext = level + (with_p ? C->K : 0);
     a.L = C->L;
     a.k_p = C->K;
     a.beta = C->beta(level);
+    a.beta_max = C->beta_max;
     a.log_n = C->log_n;
-    a.diag_level = f->level;
+    u32 packed = 0;
+    for (u32 t = 0; t < a.ext; t++) packed += packed_q(C->mods[C->gmod(level, t)]) ? 1 : 0;
+    a.wide = 2 * packed < a.ext;
     a.err = (u32*)C->d_err.p;
     a.wait_ns = C->dbg_wait_ns;
     a.starve_step = C->dbg_starve_step;
@@ -566,53 +601,53 @@ OuterLayer outer_layer(const ckks_ctx* C, const ckks_diags* f, int64_t step, u32
 // diagonal method the case (1, D, 1): the three share this schedule and give
 // identical residues for those splits.
 void sched_th(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 n2, u32 n3, cudaStream_t st,
-              K6Tile tile = K6Tile{}) {
+              u32 tile = 0) {
     const u32 N = C->N, ext = level + C->K, beta = C->beta(level);
     const int64_t s = f->stride;
     Arena ar(st, N);
     const u32 nb = std::max<u32>(1, std::max(n1 - 1, n3));  // widest batch of the key-switch phases
     u64* Y = ar.limbs(std::max<size_t>((size_t)nb * level, 2 * (C->K + 1)));
-    std::vector<u64*> A(n1, nullptr), B(n1, nullptr), Dg(n1, nullptr);
-    Dg[0] = ar.limbs((size_t)beta * ext);
-    // P c0 once (line 2), read by every middle-layer step of the first baby index: scaling jobs
-    // of the line-1 Decompose's forward launch
-    u64* c0l = ar.limbs(level);
-    std::vector<FwdJob> lift_jobs;
-    for (u32 t = 0; t < level; t++)
-        lift_jobs.push_back(FwdJob{io.c0 + (size_t)t * N, c0l + (size_t)t * N, nullptr, nullptr, nullptr,
-                                   C->lift_c[t], C->lift_sh[t], t, FWD_COPY | FWD_SCALE});
-    op_decompose(C, level, io.c1, 0, Dg[0], Y, st, &lift_jobs);  // line 1
-    for (u32 i = 1; i < n1; i++) {                     // lines 2-5 (the lift is fused)
-        const int64_t r = s * i;
-        A[i] = ar.limbs(ext);
-        B[i] = ar.limbs(ext);
-        op_ks_inner(C, level, Dg[0], key_of(C, r), C->galois(r), io.c0, 2, A[i], B[i], 0, st);
+    const bool mid = n2 > 1;
+    const u32 slots = mid ? beta + 1 : 1;  // of X_i: its digits and A_i, or A_i alone
+    std::vector<u64*> X(n1, nullptr), B(n1, nullptr);
+    for (u32 i = 0; i < n1; i++) X[i] = ar.limbs((size_t)slots * ext);
+    u64* D0 = mid ? X[0] : n1 > 1 ? ar.limbs((size_t)beta * ext) : nullptr;  // line 1's digits
+    const u32 d_slots = mid ? slots : beta;
+    // P c0 (line 2) into X_0's last slot: scaling jobs of the line-1 Decompose's forward launch
+    std::vector<FwdJob> lift;
+    lift_jobs(C, level, io.c0, X[0] + (size_t)(slots - 1) * BLK, (u64)slots * N, slots, lift);
+    if (D0) op_decompose_batch(C, level, {io.c1}, 0, {D0}, d_slots, Y, st, &lift);  // line 1
+    else launch_fwd_ntt(C->T, lift.data(), (int)lift.size(), st);  // no rotation but the outer ones
+    if (n1 > 1) {  // lines 2-5 for every i at once (the lift is fused)
+        std::vector<KsItem> es;
+        for (u32 i = 1; i < n1; i++) {
+            B[i] = ar.limbs(ext);
+            es.push_back(KsItem{D0, key_of(C, s * i), io.c0, X[i] + (size_t)(slots - 1) * BLK, B[i], C->galois(s * i), 0});
+        }
+        KsArgs k = ks_base(C, level, d_slots, slots);
+        k.x0_mode = 2;
+        op_ks_list(k, es, st);
     }
-    if (n2 > 1 && n1 > 1) {  // lines 6-7 for every i at once
+    if (mid && n1 > 1) {  // lines 6-7 for every i at once
         std::vector<const u64*> bs, tqc;
         std::vector<u64*> tq, dg;
         for (u32 i = 1; i < n1; i++) {
             bs.push_back(B[i]);
             tq.push_back(ar.limbs(level));
             tqc.push_back(tq.back());
-            Dg[i] = ar.limbs((size_t)beta * ext);
-            dg.push_back(Dg[i]);
+            dg.push_back(X[i]);
         }
         op_moddown_batch(C, level, bs, tq, Y, st);
-        op_decompose_batch(C, level, tqc, 0, dg, Y, st);
+        op_decompose_batch(C, level, tqc, 0, dg, slots, Y, st);
     }
     DiagMacArgs a = dm_base(C, level, true, f, tile);
     a.n1 = n1;
     a.n2 = n2;
     a.n3 = n3;
     a.lift0 = 1;
-    a.A[0] = io.c0;
-    a.B[0] = io.c1;
-    a.c0[0] = io.c0;
+    a.slots = slots;
     a.c1[0] = io.c1;
-    a.c0l[0] = c0l;
-    for (u32 i = 1; i < n1; i++) a.A[i] = A[i], a.B[i] = B[i];
-    for (u32 i = 0; i < n1; i++) a.Dg[i] = Dg[i];
+    for (u32 i = 0; i < n1; i++) a.X[i] = X[i], a.B[i] = B[i];
     for (u32 j = 1; j < n2; j++) {
         a.keys[j] = key_of(C, s * n1 * j);
         a.gal_mid[j] = C->galois(s * n1 * j);
@@ -644,28 +679,16 @@ void sched_th(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 
             dk.push_back(ar.limbs((size_t)beta * ext));
         }
         op_moddown_batch(C, level, us, tq, Y, st);
-        op_decompose_batch(C, level, tqc, 0, dk, Y, st);
-        for (size_t c0 = 0; c0 < ol.rotated.size(); c0 += KS_MAX_MULTI) {
-            KsMultiArgs m;
-            memset(&m, 0, sizeof(m));
-            m.count = (u32)std::min<size_t>(KS_MAX_MULTI, ol.rotated.size() - c0);
-            for (u32 c = 0; c < m.count; c++) {
-                const u32 k = ol.rotated[c0 + c];
-                m.digits[c] = dk[c0 + c];
-                m.keys[c] = key_of(C, ol.amount[k]);
-                m.x0[c] = U0[k];
-                m.gal[c] = C->galois(ol.amount[k]);
-            }
-            m.out0 = acc0;
-            m.out1 = acc1;
-            m.mods = (const ModC*)C->d_mods.p;
-            m.level = level;
-            m.ext = ext;
-            m.L = C->L;
-            m.beta = beta;
-            m.log_n = C->log_n;
-            launch_ks_multi(m, st);
+        op_decompose_batch(C, level, tqc, 0, dk, beta, Y, st);
+        std::vector<KsItem> es;
+        for (size_t c = 0; c < ol.rotated.size(); c++) {
+            const u32 k = ol.rotated[c];
+            es.push_back(KsItem{dk[c], key_of(C, ol.amount[k]), U0[k], acc0, acc1, C->galois(ol.amount[k]), 0});
         }
+        KsArgs k = ks_base(C, level, beta, 0);
+        k.sum = 1;
+        k.x0_mode = 1;
+        op_ks_list(k, es, st);
     }
     op_moddown_rescale_batch(C, level, std::vector<const u64*>{acc0, acc1}, std::vector<u64*>{io.o0, io.o1}, Y,
                              st);  // line 19
@@ -679,7 +702,7 @@ void sched_th(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 
 // that each diagonal and key word is fetched from HBM once for the batch.
 // The results are identical to per-ciphertext sched_th.
 void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const ckks_diags* f, u32 n1, u32 n2,
-                    u32 n3, cudaStream_t st, K6Tile tile = K6Tile{}) {
+                    u32 n3, cudaStream_t st, u32 tile = 0) {
     const u32 N = C->N, ext = level + C->K, beta = C->beta(level);
     const u32 nbat = (u32)ios.size();
     const size_t dig = (size_t)beta * ext;  // limbs of one digit set
@@ -687,44 +710,42 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
     Arena ar(st, N);
     const u32 nb = std::max<u32>(1, std::max(n1 - 1, n3)) * nbat;
     u64* Y = ar.limbs(std::max<size_t>((size_t)std::max(nb, nbat) * level, 2ull * nbat * (C->K + 1)));
-    u64* Aall = ar.limbs((size_t)nbat * n1 * ext);  // [b][i][ext]; i = 0 unused (lifted input)
-    u64* Ball = ar.limbs((size_t)nbat * n1 * ext);
-    u64* Dall = ar.limbs((size_t)nbat * n1 * dig);  // [b][i][beta][ext]
+    const bool mid = n2 > 1;
+    const u32 slots = mid ? beta + 1 : 1;  // of X_i: its digits and A_i, or A_i alone
+    u64* Xall = ar.limbs((size_t)nbat * n1 * slots * ext);  // [b][i][ext][N/BLK][slots][BLK]
+    u64* Ball = n1 > 1 ? ar.limbs((size_t)nbat * n1 * ext) : nullptr;  // [b][i][ext]; i = 0 unused (lifted input)
+    u64* D0 = !mid && n1 > 1 ? ar.limbs((size_t)nbat * dig) : nullptr;  // line 1's digits where X has none
     u64* Uall = ar.limbs((size_t)nbat * n3 * 2 * ext);  // [b][k][c][ext]
-    auto Ap = [&](u32 b, u32 i) { return Aall + ((size_t)b * n1 + i) * ext * N; };
+    const u32 d_slots = mid ? slots : beta;
+    auto Xp = [&](u32 b, u32 i) { return Xall + ((size_t)b * n1 + i) * slots * ext * N; };
+    auto Ap = [&](u32 b, u32 i) { return Xp(b, i) + (size_t)(slots - 1) * BLK; };
     auto Bp = [&](u32 b, u32 i) { return Ball + ((size_t)b * n1 + i) * ext * N; };
-    auto Dp = [&](u32 b, u32 i) { return Dall + ((size_t)b * n1 + i) * dig * N; };
+    auto Dp = [&](u32 b) { return mid ? Xp(b, 0) : D0 + (size_t)b * dig * N; };
     auto Up = [&](u32 b, u32 k, u32 c) { return Uall + (((size_t)b * n3 + k) * 2 + c) * ext * N; };
-    {  // line 1
+    {  // line 1, and P c0 (line 2)
         std::vector<const u64*> cs;
         std::vector<u64*> ds;
-        for (u32 b = 0; b < nbat; b++) cs.push_back(ios[b].c1), ds.push_back(Dp(b, 0));
-        op_decompose_batch(C, level, cs, 0, ds, Y, st);
+        std::vector<FwdJob> lift;
+        for (u32 b = 0; b < nbat; b++) {
+            lift_jobs(C, level, ios[b].c0, Ap(b, 0), (u64)slots * N, slots, lift);
+            cs.push_back(ios[b].c1);
+            ds.push_back(Dp(b));
+        }
+        if (mid || n1 > 1) op_decompose_batch(C, level, cs, 0, ds, d_slots, Y, st, &lift);
+        else launch_fwd_ntt(C->T, lift.data(), (int)lift.size(), st);
     }
-    if (n1 > 1) {  // lines 2-5, every (i, b) in launches of KS_MAX_BATCH products
-        std::vector<KsBatchEntry> es;
+    if (n1 > 1) {  // lines 2-5, every (i, b) in launches of KS_MAX products
+        std::vector<KsItem> es;
         for (u32 i = 1; i < n1; i++)
             for (u32 b = 0; b < nbat; b++) {
                 const int64_t r = s * i;
-                es.push_back(KsBatchEntry{Dp(b, 0), key_of(C, r), ios[b].c0, Ap(b, i), Bp(b, i), C->galois(r), 0});
+                es.push_back(KsItem{Dp(b), key_of(C, r), ios[b].c0, Ap(b, i), Bp(b, i), C->galois(r), 0});
             }
-        for (size_t e0 = 0; e0 < es.size(); e0 += KS_MAX_BATCH) {
-            KsBatchArgs k;
-            memset(&k, 0, sizeof(k));
-            k.count = (u32)std::min<size_t>(KS_MAX_BATCH, es.size() - e0);
-            for (u32 c = 0; c < k.count; c++) k.e[c] = es[e0 + c];
-            k.mods = (const ModC*)C->d_mods.p;
-            k.lift_c = C->d_lift.p;
-            k.lift_sh = C->d_lift_sh.p;
-            k.level = level;
-            k.ext = ext;
-            k.L = C->L;
-            k.beta = beta;
-            k.log_n = C->log_n;
-            launch_ks_batch(k, st);
-        }
+        KsArgs k = ks_base(C, level, d_slots, slots);
+        k.x0_mode = 2;
+        op_ks_list(k, es, st);
     }
-    if (n2 > 1 && n1 > 1) {  // lines 6-7
+    if (mid && n1 > 1) {  // lines 6-7
         std::vector<const u64*> bs, tqc;
         std::vector<u64*> tq, dg;
         for (u32 b = 0; b < nbat; b++)
@@ -732,33 +753,22 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
                 bs.push_back(Bp(b, i));
                 tq.push_back(ar.limbs(level));
                 tqc.push_back(tq.back());
-                dg.push_back(Dp(b, i));
+                dg.push_back(Xp(b, i));
             }
         op_moddown_batch(C, level, bs, tq, Y, st);
-        op_decompose_batch(C, level, tqc, 0, dg, Y, st);
+        op_decompose_batch(C, level, tqc, 0, dg, slots, Y, st);
     }
     DiagMacArgs a = dm_base(C, level, true, f, tile);
     a.n1 = n1;
     a.n2 = n2;
     a.n3 = n3;
     a.lift0 = 1;
+    a.slots = slots;
     a.batch = nbat;
-    for (u32 b = 0; b < nbat; b++) a.c0[b] = ios[b].c0, a.c1[b] = ios[b].c1;
-    {  // P c0 once per ciphertext (line 2)
-        std::vector<const u64*> cin;
-        std::vector<u64*> cout;
-        u64* c0l = ar.limbs((size_t)nbat * level);
-        for (u32 b = 0; b < nbat; b++) {
-            cin.push_back(ios[b].c0);
-            cout.push_back(c0l + (size_t)b * level * N);
-            a.c0l[b] = cout.back();
-        }
-        launch_lift((const ModC*)C->d_mods.p, C->d_lift.p, C->d_lift_sh.p, cin.data(), cout.data(), nbat, level,
-                    C->log_n, st);
-    }
-    for (u32 i = 0; i < n1; i++) a.A[i] = Ap(0, i), a.B[i] = Bp(0, i), a.Dg[i] = Dp(0, i);
-    a.bs_ab = (u64)n1 * ext * N;
-    a.bs_dg = (u64)n1 * dig * N;
+    for (u32 b = 0; b < nbat; b++) a.c1[b] = ios[b].c1;
+    for (u32 i = 0; i < n1; i++) a.X[i] = Xp(0, i), a.B[i] = i ? Bp(0, i) : nullptr;
+    a.bs_x = (u64)n1 * slots * ext * N;
+    a.bs_b = (u64)n1 * ext * N;
     a.bs_u = (u64)n3 * 2 * ext * N;
     for (u32 j = 1; j < n2; j++) {
         a.keys[j] = key_of(C, s * n1 * j);
@@ -792,29 +802,19 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
                 dk.push_back(ar.limbs(dig));
             }
         op_moddown_batch(C, level, us, tq, Y, st);
-        op_decompose_batch(C, level, tqc, 0, dk, Y, st);
-        for (u32 b = 0; b < nbat; b++)
-            for (size_t c0 = 0; c0 < nrot; c0 += KS_MAX_MULTI) {
-                KsMultiArgs m;
-                memset(&m, 0, sizeof(m));
-                m.count = (u32)std::min<size_t>(KS_MAX_MULTI, nrot - c0);
-                for (u32 c = 0; c < m.count; c++) {
-                    const u32 k = ol.rotated[c0 + c];
-                    m.digits[c] = dk[(size_t)b * nrot + c0 + c];
-                    m.keys[c] = key_of(C, ol.amount[k]);
-                    m.x0[c] = Up(b, k, 0);
-                    m.gal[c] = C->galois(ol.amount[k]);
-                }
-                m.out0 = Acc(b, 0);
-                m.out1 = Acc(b, 1);
-                m.mods = (const ModC*)C->d_mods.p;
-                m.level = level;
-                m.ext = ext;
-                m.L = C->L;
-                m.beta = beta;
-                m.log_n = C->log_n;
-                launch_ks_multi(m, st);
+        op_decompose_batch(C, level, tqc, 0, dk, beta, Y, st);
+        for (u32 b = 0; b < nbat; b++) {
+            std::vector<KsItem> es;
+            for (size_t c = 0; c < nrot; c++) {
+                const u32 k = ol.rotated[c];
+                es.push_back(KsItem{dk[(size_t)b * nrot + c], key_of(C, ol.amount[k]), Up(b, k, 0), Acc(b, 0), Acc(b, 1),
+                                    C->galois(ol.amount[k]), 0});
             }
+            KsArgs k = ks_base(C, level, beta, 0);
+            k.sum = 1;
+            k.x0_mode = 1;
+            op_ks_list(k, es, st);
+        }
     }
     std::vector<const u64*> xs;
     std::vector<u64*> outs;
@@ -830,7 +830,7 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
 // BSGS, Eq. (5): un-hoisted rotations (each with its own Decompose of the
 // rotated c1 and two ModDowns), products over Q, plain rescale at the end.
 void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 n2, cudaStream_t st,
-                K6Tile tile = K6Tile{}) {
+                u32 tile = 0) {
     const u32 N = C->N, ext = level + C->K, beta = C->beta(level);
     const int64_t s = f->stride;
     Arena ar(st, N);
@@ -857,13 +857,14 @@ void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u3
     a.n1 = n1;
     a.n2 = 1;
     a.n3 = n2;
-    a.A[0] = io.c0;
+    a.slots = 1;
+    a.X[0] = io.c0;
     a.B[0] = io.c1;
     for (u32 i = 1; i < n1; i++) {
         u64* c0 = ar.limbs(level);
         u64* c1 = ar.limbs(level);
         rotate_into(io.c0, io.c1, s * i, c0, c1, 0);
-        a.A[i] = c0;
+        a.X[i] = c0;
         a.B[i] = c1;
     }
     const OuterLayer ol = outer_layer(C, f, n1, n2);
@@ -1110,7 +1111,6 @@ ckks_status ckks_debug_diag_mac_tile(ckks_ctx* ctx, uint32_t outer_per_cta, uint
         if (positions_per_cta != 0 && positions_per_cta != 128 && positions_per_cta != 256 && positions_per_cta != 512)
             fail(CKKS_EINVAL, "positions per CTA: 0, 128, 256 or 512");
         ctx->dbg_tile_k3 = outer_per_cta;
-        ctx->dbg_tile_run = positions_per_cta;
     });
 }
 
@@ -1191,6 +1191,17 @@ ckks_status ckks_ctx_create(ckks_ctx** out, uint32_t log_n, const uint64_t* q, u
         for (u32 i = 0; i < nm; i++) {
             const u64 m = C->mods[i];
             mc[i] = modc_h(m);
+            const bool pk = packed_q(m);
+            const u64 lb = (u64)(N / BLK) * diag_blk(pk);
+            mc[i].koff = C->key_bytes;
+            C->key_bytes += (u64)(N / BLK) * key_blk(pk, C->beta_max, C->beta_max);
+            if (i < n_q) {
+                mc[i].doff = C->q_bytes.back();
+                C->q_bytes.push_back(C->q_bytes.back() + lb);
+            } else {
+                mc[i].doff = C->p_bytes;
+                C->p_bytes += lb;
+            }
             // psi = x^((m-1)/2N) for the smallest x >= 2 with psi^N = -1
             u64 w = 0;
             for (u64 x = 2;; x++) {
@@ -1250,28 +1261,40 @@ ckks_status ckks_ctx_destroy(ckks_ctx* ctx) {
     });
 }
 
+static PackArgs pack_args(const ckks_ctx* ctx, const u64* in, unsigned char* out) {
+    PackArgs p{};
+    p.in = in;
+    p.out = out;
+    p.mods = (const ModC*)ctx->d_mods.p;
+    p.L = ctx->L;
+    p.k = ctx->K;
+    p.beta_max = ctx->beta_max;
+    p.log_n = ctx->log_n;
+    return p;
+}
+
 static void put_key(ckks_ctx* ctx, int32_t r, const uint64_t* src, size_t n_words, cudaMemcpyKind kind,
                     cudaStream_t st) {
     if (!ctx || !src) fail(CKKS_EINVAL, "null argument");
     if (n_words != ctx->key_words()) fail(CKKS_EINVAL, "key size must be beta_max*2*(L+k)*N words");
     CK(cudaSetDevice(ctx->device));
     const u32 rk = ctx->rotkey(r);
-    u64* d;
+    unsigned char* d;
     auto it = ctx->keys.find(rk);
     if (it != ctx->keys.end()) d = it->second;
-    else d = ctx->dalloc(n_words);
+    else d = (unsigned char*)ctx->dalloc(ctx->key_bytes / 8);
     ctx->keys[rk] = d;
-    // stored with the two components interleaved per word (one 16-byte load per digit word)
-    const size_t plane = (size_t)(ctx->L + ctx->K) * ctx->N;
+    PackArgs p = pack_args(ctx, src, d);
     if (kind == cudaMemcpyHostToDevice) {
         u64* tmp = ctx->dalloc(n_words);
         CK(cudaMemcpy(tmp, src, n_words * 8, kind));
-        launch_interleave_key(tmp, d, plane, ctx->beta_max, 0);
+        p.in = tmp;
+        launch_pack_key(p, 0);
         CK(cudaGetLastError());
         CK(cudaDeviceSynchronize());
         ctx->dfree(tmp, n_words);
     } else {
-        launch_interleave_key(src, d, plane, ctx->beta_max, st);
+        launch_pack_key(p, st);
         CK(cudaGetLastError());
     }
 }
@@ -1287,6 +1310,18 @@ ckks_status ckks_upload_rotation_key_device(ckks_ctx* ctx, int32_t r, const uint
 
 int ckks_has_rotation_key(const ckks_ctx* ctx, int32_t r) {
     return ctx && ctx->keys.count(ctx->rotkey(r)) ? 1 : 0;
+}
+
+// Packs diagonals [first, first + count) of f from words [count][level + k][N]
+// on the device, in stream order.
+static void pack_diags(const ckks_diags* f, u32 first, u32 count, const u64* dev, cudaStream_t st) {
+    const ckks_ctx* ctx = f->ctx;
+    PackArgs p = pack_args(ctx, dev, f->d + (size_t)first * ctx->diag_bytes(f->level));
+    p.level = f->level;
+    p.p_base = ctx->q_bytes[f->level];
+    p.stride = ctx->diag_bytes(f->level);
+    launch_pack_diags(p, count, st);
+    CK(cudaGetLastError());
 }
 
 static void put_diags(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, int32_t offset0, int32_t stride,
@@ -1306,9 +1341,31 @@ static void put_diags(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, int32_t 
         f->level = level;
         f->offset0 = offset0;
         f->stride = stride;
-        f->d = ctx->dalloc(n_words);
-        if (kind == cudaMemcpyHostToDevice) CK(cudaMemcpy(f->d, host, n_words * 8, kind));
-        else CK(cudaMemcpyAsync(f->d, host, n_words * 8, kind, st));
+        const size_t words = (size_t)n_diag * ctx->diag_bytes(level) / 8;
+        f->d = (unsigned char*)ctx->dalloc(words);
+        u64* tmp = nullptr;
+        size_t tmp_words = 0;
+        try {
+            if (kind == cudaMemcpyHostToDevice) {  // through a staging buffer of at most 256 MB, or one diagonal
+                const size_t per = (size_t)(level + ctx->K) * ctx->N;
+                const u32 chunk = (u32)std::min<size_t>(n_diag, std::max<size_t>(1, (size_t(256) << 20) / (per * 8)));
+                tmp_words = per * chunk;
+                tmp = ctx->dalloc(tmp_words);
+                for (u32 d0 = 0; d0 < n_diag; d0 += chunk) {
+                    const u32 n = std::min(chunk, n_diag - d0);
+                    CK(cudaMemcpy(tmp, host + per * d0, per * n * 8, kind));
+                    pack_diags(f.get(), d0, n, tmp, 0);
+                }
+                CK(cudaDeviceSynchronize());
+                ctx->dfree(tmp, tmp_words);
+            } else {
+                pack_diags(f.get(), 0, n_diag, host, st);
+            }
+        } catch (...) {
+            if (tmp) ctx->dfree(tmp, tmp_words);
+            ctx->dfree((u64*)f->d, words);
+            throw;
+        }
         *out = f.release();
 }
 
@@ -1345,7 +1402,7 @@ ckks_status ckks_diags_create(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, 
         f->level = level;
         f->offset0 = offset0;
         f->stride = stride;
-        f->d = ctx->dalloc((size_t)n_diag * (level + ctx->K) * ctx->N);
+        f->d = (unsigned char*)ctx->dalloc((size_t)n_diag * ctx->diag_bytes(level) / 8);
         *out = f.release();
     });
 }
@@ -1358,7 +1415,7 @@ ckks_status ckks_diags_write_device(ckks_diags* f, uint32_t first, uint32_t coun
         if ((u64)first + count > f->n_diag) fail(CKKS_EINVAL, "range exceeds n_diag");
         if (n_words != per * count) fail(CKKS_EINVAL, "size mismatch");
         CK(cudaSetDevice(f->ctx->device));
-        CK(cudaMemcpyAsync(f->d + per * first, dev, n_words * 8, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
+        if (count) pack_diags(f, first, count, dev, (cudaStream_t)stream);
     });
 }
 
@@ -1366,7 +1423,7 @@ ckks_status ckks_free_diags(ckks_diags* f) {
     return guarded([&] {
         if (!f) return;
         cudaSetDevice(f->ctx->device);
-        f->ctx->dfree(f->d, (size_t)f->n_diag * (f->level + f->ctx->K) * f->ctx->N);
+        f->ctx->dfree((u64*)f->d, (size_t)f->n_diag * f->ctx->diag_bytes(f->level) / 8);
         delete f;
     });
 }
@@ -1563,22 +1620,18 @@ ckks_status lt_autotune(ckks_ctx* ctx, lt_algo algo, const ckks_ct* sample, cons
         {
             std::lock_guard<std::mutex> g(ctx->mu);
             ctx->tuned[key] = bsp;
-            ctx->tuned_tile[key] = {0u, 0u};
+            ctx->tuned_tile[key] = 0;
         }
-        // the diagonal kernel's tile for the chosen split: fewer outer indices per CTA
-        // (half the default), and the other number of positions per CTA (see launch_ws)
+        // the diagonal kernel's tile for the chosen split: half the default outer indices per CTA
         if (algo != LT_BSGS) {
             const lt_split t = th_form(ctx, level, f, algo, bsp);
             u32 k3 = 1;
             while (k3 < t.n3 && k3 < (u32)DM_MAX_K3) k3 *= 2;
-            std::vector<std::pair<u32, u32>> tiles;
-            if (k3 >= 2) tiles.push_back({k3 / 2, 0u});
-            tiles.push_back({0u, 256u});
-            std::pair<u32, u32> btile{0u, 0u};
-            for (const auto& tl : tiles) {
+            u32 btile = 0;
+            if (k3 >= 2) {
                 {
                     std::lock_guard<std::mutex> g(ctx->mu);
-                    ctx->tuned_tile[key] = tl;
+                    ctx->tuned_tile[key] = k3 / 2;
                 }
                 lt_eval_impl(ctx, sample, f, algo, &bsp, out, st, nullptr);
                 CK(cudaEventRecord(e0, st));
@@ -1588,7 +1641,7 @@ ckks_status lt_autotune(ckks_ctx* ctx, lt_algo algo, const ckks_ct* sample, cons
                 CK(cudaEventSynchronize(e1));
                 float ms = 0;
                 CK(cudaEventElapsedTime(&ms, e0, e1));
-                if (ms / reps < best) best = ms / reps, btile = tl;
+                if (ms / reps < best) best = ms / reps, btile = k3 / 2;
             }
             std::lock_guard<std::mutex> g(ctx->mu);
             ctx->tuned_tile[key] = btile;
@@ -1682,8 +1735,8 @@ int32_t lt_tuned_tile(const ckks_ctx* ctx, lt_algo algo, const ckks_diags* f, ui
     auto tt = ctx->tuned_tile.find(
         std::make_tuple((int)algo, level, f->n_diag, f->stride, (int32_t)ctx->rotkey(f->offset0)));
     if (tt == ctx->tuned_tile.end()) return 0;
-    *outer_per_cta = tt->second.first;
-    *positions_per_cta = tt->second.second;
+    *outer_per_cta = tt->second;
+    *positions_per_cta = 0;
     return 1;
 }
 
@@ -1743,21 +1796,21 @@ static lt_split th_form(const ckks_ctx* ctx, u32 level, const ckks_diags* f, lt_
 
 // The diagonal kernel's tile for an LT: the one lt_autotune measured for the
 // shape when `sp` is the shape's tuned split, else the default.
-static K6Tile tile_for(const ckks_ctx* ctx, u32 level, const ckks_diags* f, lt_algo algo, const lt_split& sp) {
+static u32 tile_for(const ckks_ctx* ctx, u32 level, const ckks_diags* f, lt_algo algo, const lt_split& sp) {
     std::lock_guard<std::mutex> g(ctx->mu);
-    if (ctx->dbg_tile_k3 || ctx->dbg_tile_run) return K6Tile{ctx->dbg_tile_k3, ctx->dbg_tile_run};
+    if (ctx->dbg_tile_k3) return ctx->dbg_tile_k3;
     const auto key = std::make_tuple((int)algo, level, f->n_diag, f->stride, (int32_t)ctx->rotkey(f->offset0));
     auto it = ctx->tuned.find(key);
     auto tt = ctx->tuned_tile.find(key);
-    if (it == ctx->tuned.end() || tt == ctx->tuned_tile.end()) return K6Tile{};
+    if (it == ctx->tuned.end() || tt == ctx->tuned_tile.end()) return 0;
     const lt_split& t = it->second;
-    if (t.n1 != sp.n1 || t.n2 != sp.n2 || (algo == LT_TH_BSGS && t.n3 != sp.n3)) return K6Tile{};
-    return K6Tile{tt->second.first, tt->second.second};
+    if (t.n1 != sp.n1 || t.n2 != sp.n2 || (algo == LT_TH_BSGS && t.n3 != sp.n3)) return 0;
+    return tt->second;
 }
 
 static void dispatch(ckks_ctx* ctx, u32 level, const LtIO& io, const ckks_diags* f, lt_algo algo, const lt_split& sp,
                      cudaStream_t st) {
-    const K6Tile tile = tile_for(ctx, level, f, algo, sp);
+    const u32 tile = tile_for(ctx, level, f, algo, sp);
     if (algo == LT_BSGS) {
         sched_bsgs(ctx, level, io, f, sp.n1, sp.n2, st, tile);
         return;
@@ -1854,7 +1907,7 @@ ckks_status lt_eval_batch(ckks_ctx* ctx, uint32_t count, const ckks_ct* const* i
                 done[b] = true;
             }
             const ckks_diags* fa = f[ia.idx];
-            const K6Tile tile = tile_for(ctx, lva, fa, ia.algo, ia.sp);
+            const u32 tile = tile_for(ctx, lva, fa, ia.algo, ia.sp);
             units.push_back(Unit{one * group.size(), [=](cudaStream_t s) {
                                      sched_th_batch(ctx, lva, group, fa, n1, n2, n3, s, tile);
                                  }});

@@ -8,6 +8,39 @@
 
 namespace ckks {
 
+// ------------------------------------------------------------------ layout of keys and diagonals
+// Switching keys and diagonals are what an LT streams from HBM, so the library
+// stores them at 5 bytes a word where the modulus allows it (2^32 < q < 2^40:
+// 23 of the 28 limbs of the N = 2^16 workload, 31% fewer bytes) and at 8 bytes
+// otherwise.  A limb is stored in blocks of BLK = 128 consecutive words, the
+// unit that every automorphism maps onto one block (Eq. 8), so that one bulk
+// copy fetches a block:
+//   diagonals : packed  [128 x u32 low words][128 x u8 high bytes], 640 bytes
+//               wide    [128 x u64], 1024 bytes
+//   keys      : packed  [128 x key_hi bytes: the high bytes of (component 0, component 1) per digit]
+//                       [beta_max][128 x (u32, u32) low words]
+//               wide    [beta_max][128 x (u64, u64)]
+// A level with beta < beta_max digits reads a prefix of a key block.
+constexpr u32 BLK = 128;
+__host__ __device__ inline bool packed_q(u64 q) { return q > (1ull << 32) && q < (1ull << 40); }
+__host__ __device__ inline u32 diag_blk(bool packed) { return packed ? BLK * 5 : BLK * 8; }
+__host__ __device__ inline u32 key_hi(u32 beta_max) { return (2 * beta_max + 3) & ~3u; }  // bytes per position
+// bytes of the first beta digits of a key block (beta = beta_max: of the block)
+__host__ __device__ inline u32 key_blk(bool packed, u32 beta, u32 beta_max) {
+    return packed ? BLK * (key_hi(beta_max) + 8 * beta) : BLK * 16 * beta;
+}
+// Words [rows][N] -> packed or wide limbs, reduced on the way, so that any word
+// of the residue class is taken.
+struct PackArgs {
+    const u64* in;
+    unsigned char* out;
+    const ModC* mods;
+    u32 level, L, k, beta_max, log_n;  // diagonals: Q limbs stored; keys: beta_max
+    u64 p_base, stride;                // diagonals: offset of the P limbs, bytes per diagonal
+};
+void launch_pack_diags(const PackArgs& a, u32 count, cudaStream_t st);
+void launch_pack_key(const PackArgs& a, cudaStream_t st);
+
 // Per-context device tables every NTT kernel reads.
 struct NttTables {
     const ModC* mods;          // [n_mod] {q, mu}
@@ -29,8 +62,11 @@ struct NttTables {
 // unchanged; it rides in the same launch as the transforms.
 // Bit 18 (with bit 17): a scaling job instead, dst[x] = src[x] * c mod q
 // (c_sh its Shoup companion), e.g. the lift P c0 of Alg. 2 line 2.
+// Bits 19..31: the blocks of BLK words from one of dst's blocks to the next
+// (0: 1, a plain limb), for limbs that are slots of grouped blocks (DigLayout).
 constexpr u32 FWD_COPY = 1u << 17;
 constexpr u32 FWD_SCALE = 1u << 18;
+constexpr u32 FWD_STEP = 19;
 struct FwdJob {
     const u64* src;
     u64* dst;
@@ -71,63 +107,45 @@ struct AddJob {
 void launch_add_gather(const ModC* mods, const AddJob* jobs, int njobs, u32 gal, int accumulate, u32 log_n,
                        cudaStream_t st);
 
-// Switching-key inner product with hoisted automorphism (K4).
-struct KsArgs {
-    const u64* digits;      // [beta][ext][N]
-    const u64* key;         // [beta_max][L+k][N] word pairs (interleaved layout below)
-    const u64* x0;          // null, ext poly, or Q poly to lift
-    u64* out0;
-    u64* out1;
-    const ModC* mods;       // context moduli (index = global modulus id)
-    const u64* lift_c;      // [L+k] [P]_{q_j} (0 for P moduli) and Shoup companions
-    const u64* lift_sh;
-    u32 level, ext, L, beta, beta_max, gal, x0_mode, accumulate, log_n;
+// Where word x of digit b of limb t lies: t limb + (x / BLK) blk + b dig + x % BLK.
+// Plain digits [beta][ext][N], or grouped [ext][N/BLK][slots][BLK]: the slots
+// of one block side by side, so that the diagonal kernel fetches every digit
+// of a run (and the A run, the last slot) with one bulk copy.
+struct DigLayout {
+    u64 limb, blk, dig;
 };
-void launch_ks_inner(const KsArgs& a, cudaStream_t st);
+inline DigLayout plain_digits(u32 ext, u32 log_n) { return {1ull << log_n, BLK, (u64)ext << log_n}; }
+inline DigLayout grouped_digits(u32 slots, u32 log_n) { return {(u64)slots << log_n, (u64)slots * BLK, BLK}; }
 
-// out_c += sum_k phi_{r_k}(x0_k (c = 0 only) + <D_k, swk~_{r_k, c}>), k < count:
-// the outer key-switch layer of Algorithm 2 (lines 17-18) for every giant
-// index at once.
-constexpr int KS_MAX_MULTI = 64;
-struct KsMultiArgs {
-    const u64* digits[KS_MAX_MULTI];  // [beta][ext][N] each
-    const u64* keys[KS_MAX_MULTI];    // [beta_max][L+k][N] word pairs each (interleaved)
-    const u64* x0[KS_MAX_MULTI];      // [ext][N] each
-    u32 gal[KS_MAX_MULTI];
-    u64* out0;
-    u64* out1;
-    const ModC* mods;
-    u32 count, level, ext, L, beta, log_n;
-};
-void launch_ks_multi(const KsMultiArgs& a, cudaStream_t st);
-
-// Rotation keys in the library's layout: the user's [beta_max][2][L+k][N]
-// with the two components interleaved per word, [beta_max][L+k][N] x 2.
-// Every kernel that reads a key reads one 16-byte word per (digit, limb,
-// position).  plane = (L+k) N.
-void launch_interleave_key(const u64* in, u64* out, size_t plane, u32 beta_max, cudaStream_t st);
-
-// Many independent K4 products (overwrite form, x0 lifted from a Q
-// polynomial) in one launch: entry e reads digits, key and x0 and writes
-// out0/out1.  Entries that share a key are adjacent in the grid.
-constexpr int KS_MAX_BATCH = 128;
-struct KsBatchEntry {
-    const u64* digits;
-    const u64* key;
+// Switching-key inner products with hoisted automorphism (K4): for product e
+//   P_{e,c} = phi_g(x0_e) (c = 0 only) + <phi_g(d_e), swk_{e,c}>
+// x0_mode 0: no x0; 1: an extended polynomial; 2: a Q polynomial lifted to P x0.
+// sum = 0: out_{e,c} = P_{e,c}, added to what out holds if accumulate (one
+// launch for many independent products; neighbours in the grid take the same
+// run of positions, so entries that share a key read it once).
+// sum = 1: out_{0,c} += sum_e P_{e,c}, the outer key-switch layer of Algorithm
+// 2 (lines 17-18) for every giant index at once.
+constexpr int KS_MAX = 32;  // 1.5 KB of kernel parameters: every launch copies them
+struct KsItem {
+    const u64* digits;         // dl
+    const unsigned char* key;  // layout above
     const u64* x0;
-    u64* out0;
-    u64* out1;
+    u64* out0;                 // o_limb, o_blk: its limb and block strides
+    u64* out1;                 // plain
     u32 gal;
     u32 pad;
 };
-struct KsBatchArgs {
-    KsBatchEntry e[KS_MAX_BATCH];
-    const ModC* mods;
-    const u64* lift_c;
+struct KsArgs {
+    KsItem e[KS_MAX];
+    const ModC* mods;  // context moduli (index = global modulus id)
+    const u64* lift_c; // [L+k] [P]_{q_j} (0 for P moduli) and Shoup companions
     const u64* lift_sh;
-    u32 count, level, ext, L, beta, log_n;
+    u32* err;          // set to nonzero when a bounded device wait gives up
+    DigLayout dl;
+    u64 o_limb, o_blk;
+    u32 count, sum, x0_mode, accumulate, level, ext, L, beta, beta_max, log_n;
 };
-void launch_ks_batch(const KsBatchArgs& a, cudaStream_t st);
+void launch_ks(const KsArgs& a, cudaStream_t st);
 
 // Multi-output plaintext-diagonal multiply-accumulate with the middle
 // (hoisted) key-switch layer fused in (K6).  See ks.cu.
@@ -140,17 +158,21 @@ struct DiagMacArgs {
     const ModC* mods;
     const u64* lift_c;
     const u64* lift_sh;
-    const u64* diags;       // [n_diag][diag_level + k][N]
-    const u64* A[DM_MAX_N1];
-    const u64* B[DM_MAX_N1];
-    const u64* Dg[DM_MAX_N1];        // digits per baby index (middle layer), [beta][ext][N]
-    const u64* keys[DM_MAX_N2];      // middle-layer keys, index j (j >= 1)
+    const unsigned char* diags;  // [n_diag] of diag_stride bytes, the P limbs at diag_p
+    u64 diag_stride, diag_p;
+    const u64* X[DM_MAX_N1];         // per baby index: its digits and A_i, [ext][N/BLK][slots][BLK], A_i the last slot
+    const u64* B[DM_MAX_N1];         // B_i [ext][N] (i = 0 with lift0: c1 below)
+    const unsigned char* keys[DM_MAX_N2];  // middle-layer keys, index j (j >= 1)
     u32 gal_mid[DM_MAX_N2];          // x -> x^gal for rotation n1*j*stride
     u64* U0[DM_MAX_N3];
     u64* U1[DM_MAX_N3];
     u32 gal_diag[DM_MAX_N3];         // rotation -(n1*n2*k*stride), 0 = none
-    u32 level, ext, L, k_p, beta, log_n;
-    u32 n1, n2, n3, lift0, diag_level;
+    u32 level, ext, L, k_p, beta, beta_max, log_n;
+    u32 n1, n2, n3;
+    u32 slots;                       // beta + 1, or 1 without a middle layer (n2 = 1)
+    // 1: (A_0, B_0) is the lifted input P (c0, c1) (Alg. 2 line 2), zero on
+    // the P limbs; X[0] holds P c0 on the Q limbs, c1 is lifted here
+    u32 lift0;
     u32* err;                        // set to nonzero when a bounded device wait gives up
     // Failure-detection test hook of the staged kernel: the step loop's
     // waits give up after wait_ns (0: the default of one second), and step
@@ -158,28 +180,23 @@ struct DiagMacArgs {
     // The drain of copies in flight always keeps the default limit.
     u64 wait_ns;
     u32 starve_step;
-    // Tile (0 = default): outer indices per CTA (a power of two below the
-    // default, which is the next power of two >= n3, at most 8) and positions
-    // per CTA (128, 256 or 512; see launch_ws).  Results do not depend on it.
-    u32 tile_k3, tile_run;
+    // Tile (0 = default): outer indices per CTA, a power of two below the
+    // next power of two >= n3, at most 8.  Results do not depend on it.
+    u32 tile_k3;
+    u32 wide;  // most limbs are wide (not packed_q)
     // Batch of ciphertexts sharing the diagonals and keys: ciphertext b uses
-    // c0[b], c1[b] as its lifted inputs and A[i] + b*bs_ab, B[i] + b*bs_ab,
-    // Dg[i] + b*bs_dg, U0/U1[k] + b*bs_u for the rest.  CTAs of the same
-    // (limb, run) for different b are adjacent in the grid, so the diagonal
-    // and key words they share are read from HBM once.
+    // X[i] + b*bs_x, B[i] + b*bs_b, c1[b] and U0/U1[k] + b*bs_u.  CTAs of the
+    // same (limb, run) for different b are adjacent in the grid, so the
+    // diagonal and key words they share are read from HBM once.
     u32 batch;
-    u64 bs_ab, bs_dg, bs_u;
-    const u64* c0[DM_MAX_B];
+    u64 bs_x, bs_b, bs_u;
     const u64* c1[DM_MAX_B];
-    // P c0 per ciphertext (Q limbs [level][N], from launch_lift), or null:
-    // the lifted input of Alg. 2 line 2 computed once instead of at every step
-    const u64* c0l[DM_MAX_B];
 };
 void launch_diag_mac(const DiagMacArgs& a, cudaStream_t st);
-// out_i[t][s] = in_i[t][s] * [P]_{q_t} mod q_t for t < level (Alg. 2 line 2,
-// the Q limbs of P c0; the P limbs are zero and not stored), i < count.
-void launch_lift(const ModC* mods, const u64* lift_c, const u64* lift_sh, const u64* const* in, u64* const* out,
-                 u32 count, u32 level, u32 log_n, cudaStream_t st);
+// Its staged kernel with K3 (1, 2, 4 or 8) outer indices per CTA and MINB CTAs
+// per SM, or false if a shape does not fit (diag_mac.cuh).
+template <int K3, int MINB>
+bool launch_ws(const DiagMacArgs& a, cudaStream_t st);
 void launch_wait_selftest(u32* err, u64 limit_ns, cudaStream_t st);
 
 uint64_t launches();

@@ -290,6 +290,14 @@ __device__ __forceinline__ void gs_s(u64& a, u64& b, const ulonglong2& t, u64 q)
 // conflicts.
 __device__ __forceinline__ u32 pad16(u32 i) { return i + (i >> 4); }
 
+// Offset of word row * C + col of a limb whose blocks of BLK words lie step words apart.
+template <u32 C>
+__device__ __forceinline__ u32 blk_off(u32 row, u32 col, u32 step) {
+    if constexpr (C >= BLK) return (row * (C / BLK) + col / BLK) * step + col % BLK;
+    else return row / (BLK / C) * step + row % (BLK / C) * C + col;
+}
+__device__ __forceinline__ u32 fwd_step(const FwdJob& J) { return max(1u, J.nsrc >> FWD_STEP) * BLK; }
+
 // ------------------------------------------------------------------ forward, column pass
 // Global stages 0..LOGS-1 (m = 2^ss, twiddle psi^brv(m + r / 2t_r)).
 template <int LOGS, bool GROW>
@@ -374,6 +382,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_fwd_cols(const __grid_constant__
     const ModC m = T.mods[J.mod];
     const u64 q = m.q;
     const ulonglong2* tw = T.psi + (size_t)J.mod * N;
+    const u32 step = fwd_step(J);
     if (J.nsrc & FWD_COPY) {  // a pass-through limb: the block copies its columns (every word loaded first)
         u64 y[16];
         if (J.nsrc & FWD_SCALE) {
@@ -388,7 +397,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_fwd_cols(const __grid_constant__
             }
         }
 #pragma unroll
-        for (int v = 0; v < 16; v++) J.dst[(size_t)(u + TPL * v) * C + col] = y[v];
+        for (int v = 0; v < 16; v++) J.dst[blk_off<C>(u + TPL * v, col, step)] = y[v];
         return;
     }
     // the S - 1 twiddle pairs of the column stages (indices 1 .. S - 1), copied while the words load
@@ -426,7 +435,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_fwd_cols(const __grid_constant__
     if (q < FWD_GROW_MAX) fwd_cols_stages<LOGS, true>(x, sm, u, c, ts, q);
     else fwd_cols_stages<LOGS, false>(x, sm, u, c, ts, q);
 #pragma unroll
-    for (int v = 0; v < 16; v++) J.dst[(size_t)(16 * u + v) * C + col] = x[v];
+    for (int v = 0; v < 16; v++) J.dst[blk_off<C>(16 * u + v, col, step)] = x[v];
 }
 
 // ------------------------------------------------------------------ forward, row pass
@@ -490,9 +499,10 @@ __device__ __forceinline__ void fwd_rows_limb(const FwdJob& J, const ModC& m, co
     constexpr u32 S = 1u << LOGS, TPL = S / 16, log_r = LOGN - LOGS;
     const u64 q = m.q;
     const size_t base = (size_t)row * S;
+    const u32 step = SUBMUL ? BLK : fwd_step(J);  // a ModDown's limbs are plain
     u64 x[16];
 #pragma unroll
-    for (int v = 0; v < 16; v++) x[v] = J.dst[base + u + TPL * v];
+    for (int v = 0; v < 16; v++) x[v] = J.dst[blk_off<S>(row, u + TPL * v, step)];
     cp_async_wait_all();
     __syncwarp();  // a row's threads are lanes of one warp
     fwd_rows_stages<LOGS, (AR > 0)>(x, sr, u, row, log_r, tw, q, t1);
@@ -527,7 +537,7 @@ __device__ __forceinline__ void fwd_rows_limb(const FwdJob& J, const ModC& m, co
         if constexpr (SUBMUL) {
             J.subout[base + xi] = mul_shoup(sub_mod(sx[v], val, q), J.c, J.c_sh, q);
         } else {
-            J.dst[base + xi] = val;
+            J.dst[blk_off<S>(row, xi, step)] = val;
         }
     }
 }
@@ -736,6 +746,7 @@ void fwd_impl(const NttTables& T, const Jobs<FwdJob>& p, int n, bool bconv, bool
         else k_fwd_cols<LR + LC, LR, false><<<g1, THREADS, 0, st>>>(T, p);
     }
     {
+        if (!nt) return;  // copies only
         ProfScope ps(K_FWD_ROWS, st, 0, half * LC);
         constexpr size_t sm = fwd_rows_smem<LC>();
         static std::atomic<uint64_t> lim_t{0}, lim_f{0};
@@ -832,16 +843,17 @@ __global__ void __launch_bounds__(PROBE_THREADS, 4) k_probe_bfly(const ulonglong
 void launch_fwd_ntt(const NttTables& T, const FwdJob* jobs, int njobs, cudaStream_t st) {
     if (njobs <= 0) return;
     // every transform job of a launch is of one kind (copy jobs may join any)
-    bool bconv = false, submul = false;
+    bool bconv = false, submul = false, transforms = false;
     for (int i = 0; i < njobs; i++)
         if (!(jobs[i].nsrc & FWD_COPY)) {
             bconv = (jobs[i].nsrc & 0xFFFFu) > 0;
+            transforms = true;
             submul = jobs[i].subout != nullptr;
             break;
         }
     for_chunks(jobs, njobs, [&](const Jobs<FwdJob>& p, int n) {
         NTT_DISPATCH(fwd_impl, bconv, submul);
-        count_launch(2);
+        count_launch(transforms ? 2 : 1);
     });
 }
 
