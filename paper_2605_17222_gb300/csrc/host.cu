@@ -387,9 +387,9 @@ void op_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& c
         u64* Yp = Y + (size_t)p * level * N;
         for (u32 b = 0; b < beta; b++) {
             const u32 first = b * C->alpha, n = std::min(C->alpha, level - first);
-            // the digit's words are canonical residues of its moduli: below 2^41 if every one is
+            // the digit's words are canonical residues of its moduli: below 2^40 if every one is
             bool small = true;
-            for (u32 j = first; j < first + n; j++) small = small && C->mods[j] < (1ull << 41);
+            for (u32 j = first; j < first + n; j++) small = small && C->mods[j] < (1ull << 40);
             for (u32 t = 0; t < ext; t++) {
                 if (t >= first && t < first + n) continue;
                 fj.push_back(FwdJob{Yp + (size_t)first * N, digits[p] + b * dl.dig + t * dl.limb,

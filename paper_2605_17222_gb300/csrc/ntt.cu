@@ -23,6 +23,7 @@
 #include <atomic>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 namespace ckks {
@@ -296,6 +297,19 @@ __device__ __forceinline__ u32 blk_off(u32 row, u32 col, u32 step) {
     if constexpr (C >= BLK) return (row * (C / BLK) + col / BLK) * step + col % BLK;
     else return row / (BLK / C) * step + row % (BLK / C) * C + col;
 }
+// Row v of a thread's consecutive rows 16 u + v in such a limb (col < C): a
+// pointer that walks the rows, so that the addresses cost adds and not the
+// multiplies the butterflies wait for.
+template <u32 C>
+__device__ __forceinline__ void next_row(u64*& p, int v, u32 step) {
+    if constexpr (C >= BLK) p += (C / BLK) * step;
+    else p += (v % (BLK / C) == BLK / C - 1) ? step - (BLK - C) : C;
+}
+// Word u + TPL v of a row (u < TPL <= 16): the offset from word u.
+template <u32 TPL>
+__device__ __forceinline__ u32 row_off(int v, u32 step) {
+    return TPL * v / BLK * step + TPL * v % BLK;
+}
 __device__ __forceinline__ u32 fwd_step(const FwdJob& J) { return max(1u, J.nsrc >> FWD_STEP) * BLK; }
 
 // ------------------------------------------------------------------ forward, column pass
@@ -326,22 +340,22 @@ __device__ __forceinline__ void fwd_cols_stages(u64 (&x)[16], u64* sm, u32 u, u3
     }
 }
 
-// Basis conversion (Eq. 3) of a column-pass thread's 16 words, NS source
-// limbs known at compile time (the constants held in registers), staged
-// through the thread's own slots of the exchange buffer.  SMALL: sources and
-// target below 2^41 (and the target above 2^32), so the four-term sums stay
-// in 96 bits (mac96) and are reduced to [0, 3q) by a fold below 2^64 and a
-// 32-bit quotient estimate (mu = floor(2^64 / q)); otherwise 128-bit sums
-// reduced lazily to [0, 4q).  Either range feeds the butterflies.
-template <int LOGS, int NS, bool SMALL>
-__device__ __forceinline__ void bconv_words(u64* sm, const FwdJob& J, u32 u, u32 c, u32 col, u32 N, u32 C,
-                                            const ModC& m) {
+// Basis conversion (Eq. 3) of a column-pass thread's 16 words, staged through
+// the thread's own slots of the exchange buffer: NS sources below 2^40, a
+// packed_q target, the constants held in registers.  The sums stay in 96 bits
+// and are reduced to [0, 3q) by a fold below 2^64 and a 32-bit quotient
+// estimate (mu = floor(2^64 / q)): for four sources the split sums of
+// bconv_words save four multiplier slots and pay as many in their second
+// reduction (level-24 LT at N = 2^16, its four column passes: 397 us, 417 with them).
+template <int LOGS, int NS>
+__device__ __forceinline__ void bconv_words96(u64* sm, const FwdJob& J, u32 u, u32 c, u32 col, u32 N, u32 C,
+                                              const ModC& m) {
     constexpr u32 S = 1u << LOGS, TPL = S / 16, W = THREADS / TPL;
     u64 cst[NS];
 #pragma unroll
     for (int j = 0; j < NS; j++) cst[j] = J.bcst[j];
     const u64 q = m.q;
-    const u64 c64 = 0 - q * m.mu_hi;                     // 2^64 mod q (mu_hi = floor(2^64 / q))
+    const u64 c64 = 0 - q * m.mu_hi;                    // 2^64 mod q (mu_hi = floor(2^64 / q))
     const u64 c63 = (c64 + ((c64 & 1) ? q : 0)) >> 1;   // 2^63 mod q
     const u32 mu32 = (u32)m.mu_hi;
     const u64* src = J.src + (size_t)u * C + col;
@@ -351,21 +365,86 @@ __device__ __forceinline__ void bconv_words(u64* sm, const FwdJob& J, u32 u, u32
         u64 y[NS];
 #pragma unroll
         for (int j = 0; j < NS; j++) y[j] = p[(size_t)j * N];
-        u64 r;
-        if constexpr (SMALL) {
-            U96 acc{0, 0};
+        U96 acc{0, 0};
 #pragma unroll
-            for (int j = 0; j < NS; j++) mac96(acc, y[j], cst[j]);
-            const u64 f = (acc.lo & ~(1ull << 63)) + ((acc.lo >> 63) ? c63 : 0) + (u64)acc.hi * c64;
-            const u64 qe = ((u64)(u32)(f >> 32) * mu32 + __umulhi((u32)f, mu32)) >> 32;
-            r = f - qe * q;
-        } else {
-            U128 acc{0, 0};
+        for (int j = 0; j < NS; j++) mac96(acc, y[j], cst[j]);
+        const u64 f = (acc.lo & ~(1ull << 63)) + ((acc.lo >> 63) ? c63 : 0) + (u64)acc.hi * c64;
+        const u64 qe = ((u64)(u32)(f >> 32) * mu32 + __umulhi((u32)f, mu32)) >> 32;
+        sm[(u + TPL * v) * W + c] = f - qe * q;
+    }
+}
+
+// The same for any sources and targets.  NS: source limbs (the constants held
+// split in registers), or 0 for any number (ns), eight to a reduction and four
+// words at a time, so that a small launch waits for four words' loads at once
+// (N = 2^14 BSGS, 44 column passes: 1014 -> 734 us).  SMALL: sources below 2^40 and a packed_q target,
+// 40-bit sums reduced to [0, 3q); otherwise 60-bit sums, reduced below 5q and
+// brought into [0, 3q).  Either feeds the butterflies.
+template <int LOGS, int NS, bool SMALL>
+__device__ __forceinline__ void bconv_words(u64* sm, const FwdJob& J, u32 ns, u32 u, u32 c, u32 col, u32 N, u32 C,
+                                            const ModC& m) {
+    constexpr u32 S = 1u << LOGS, TPL = S / 16, W = THREADS / TPL, G = NS ? NS : 8;
+    typedef typename std::conditional<SMALL, Sum40, Sum60>::type Sum;
+    const u64 q = m.q;
+    const u64* src = J.src + (size_t)u * C + col;
+    u32 k0[NS ? NS : 1], k1[NS ? NS : 1];
+    auto split_k = [](u64 x, u32& lo, u32& hi) {
+        if constexpr (SMALL) lo = (u32)x, hi = (u32)(x >> 32);
+        else split30(x, lo, hi);
+    };
+    auto split_d = [](u64 x, u32& lo, u32& hi) {
+        if constexpr (SMALL) split20(x, lo, hi);
+        else split30(x, lo, hi);
+    };
+    auto value = [&](const Sum& s, u64 add) {
+        if constexpr (SMALL) return s.value(add, q, (u32)m.mu_hi);
+        else return s.value(add, m);
+    };
 #pragma unroll
-            for (int j = 0; j < NS; j++) mac128(acc, y[j], cst[j]);
-            r = reduce128_lazy(acc, m);
+    for (int j = 0; j < NS; j++) split_k(J.bcst[j], k0[j], k1[j]);
+    // words per step: four where the sources are counted at run time, else one, unrolled four deep
+    constexpr int VG = NS ? 1 : 4, VU = NS ? 4 : 1;
+#pragma unroll VU
+    for (int v0 = 0; v0 < 16; v0 += VG) {
+        u64 r[VG] = {};
+        for (u32 j0 = 0; j0 < (NS ? 1u : ns); j0 += G) {
+            Sum s[VG];
+            if constexpr (NS > 0) {
+                u64 y[VG][NS];
+#pragma unroll
+                for (int v = 0; v < VG; v++)
+#pragma unroll
+                    for (int j = 0; j < NS; j++) y[v][j] = src[(size_t)(TPL * (v0 + v)) * C + (size_t)j * N];
+#pragma unroll
+                for (int v = 0; v < VG; v++)
+#pragma unroll
+                    for (int j = 0; j < NS; j++) {
+                        u32 d0, d1;
+                        split_d(y[v][j], d0, d1);
+                        s[v].mac(d0, d1, k0[j], k1[j]);
+                    }
+            } else {
+                const u32 je = min(j0 + G, ns);
+#pragma unroll 2
+                for (u32 j = j0; j < je; j++) {
+                    u32 c0, c1;
+                    split_k(J.bcst[j], c0, c1);
+#pragma unroll
+                    for (int v = 0; v < VG; v++) {
+                        u32 d0, d1;
+                        split_d(src[(size_t)(TPL * (v0 + v)) * C + (size_t)j * N], d0, d1);
+                        s[v].mac(d0, d1, c0, c1);
+                    }
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < VG; v++) r[v] = value(s[v], r[v]);
         }
-        sm[(u + TPL * v) * W + c] = r;
+#pragma unroll
+        for (int v = 0; v < VG; v++) {
+            if constexpr (!SMALL) r[v] = r[v] >= 2 * q ? r[v] - 2 * q : r[v];
+            sm[(u + TPL * (v0 + v)) * W + c] = r[v];
+        }
     }
 }
 
@@ -408,19 +487,13 @@ __global__ void __launch_bounds__(THREADS, 4) k_fwd_cols(const __grid_constant__
         // basis conversion (Eq. 3) of the thread's 16 words, staged through its
         // own slots of the exchange buffer so that this part stays a compact loop
         const u32 ns = J.nsrc & 0xFFFFu;
-        const bool small = ((J.nsrc >> 16) & 1u) && q > (1ull << 32) && q < (1ull << 41);
-        if (ns == 4 && small) bconv_words<LOGS, 4, true>(sm, J, u, c, col, N, C, m);
-        else if (ns == 4) bconv_words<LOGS, 4, false>(sm, J, u, c, col, N, C, m);
-        else if (ns == 5) bconv_words<LOGS, 5, false>(sm, J, u, c, col, N, C, m);
-        else {
-            const u64* bc = J.bcst;
-#pragma unroll 4
-            for (int v = 0; v < 16; v++) {
-                const u64* src = J.src + (size_t)(u + TPL * v) * C + col;
-                U128 acc{0, 0};
-                for (u32 j = 0; j < ns; j++) mac128(acc, src[(size_t)j * N], bc[j]);
-                sm[(u + TPL * v) * W + c] = reduce128_lazy(acc, m);  // [0, 4q): both butterfly forms take it
-            }
+        if (((J.nsrc >> 16) & 1u) && packed_q(q)) {
+            if (ns == 4) bconv_words96<LOGS, 4>(sm, J, u, c, col, N, C, m);
+            else bconv_words<LOGS, 0, true>(sm, J, ns, u, c, col, N, C, m);
+        } else if (ns == 4) {
+            bconv_words<LOGS, 4, false>(sm, J, ns, u, c, col, N, C, m);
+        } else {
+            bconv_words<LOGS, 0, false>(sm, J, ns, u, c, col, N, C, m);
         }
 #pragma unroll
         for (int v = 0; v < 16; v++) x[v] = sm[(u + TPL * v) * W + c];
@@ -434,8 +507,12 @@ __global__ void __launch_bounds__(THREADS, 4) k_fwd_cols(const __grid_constant__
     // and the row pass ends below 68q < 2^64 (q < 2^57)
     if (q < FWD_GROW_MAX) fwd_cols_stages<LOGS, true>(x, sm, u, c, ts, q);
     else fwd_cols_stages<LOGS, false>(x, sm, u, c, ts, q);
+    u64* p = J.dst + blk_off<C>(16 * u, col, step);
 #pragma unroll
-    for (int v = 0; v < 16; v++) J.dst[blk_off<C>(16 * u + v, col, step)] = x[v];
+    for (int v = 0; v < 16; v++) {
+        *p = x[v];
+        next_row<C>(p, v, step);
+    }
 }
 
 // ------------------------------------------------------------------ forward, row pass
@@ -500,9 +577,10 @@ __device__ __forceinline__ void fwd_rows_limb(const FwdJob& J, const ModC& m, co
     const u64 q = m.q;
     const size_t base = (size_t)row * S;
     const u32 step = SUBMUL ? BLK : fwd_step(J);  // a ModDown's limbs are plain
+    u64* p = J.dst + blk_off<S>(row, u, step);
     u64 x[16];
 #pragma unroll
-    for (int v = 0; v < 16; v++) x[v] = J.dst[blk_off<S>(row, u + TPL * v, step)];
+    for (int v = 0; v < 16; v++) x[v] = p[row_off<TPL>(v, step)];
     cp_async_wait_all();
     __syncwarp();  // a row's threads are lanes of one warp
     fwd_rows_stages<LOGS, (AR > 0)>(x, sr, u, row, log_r, tw, q, t1);
@@ -537,7 +615,7 @@ __device__ __forceinline__ void fwd_rows_limb(const FwdJob& J, const ModC& m, co
         if constexpr (SUBMUL) {
             J.subout[base + xi] = mul_shoup(sub_mod(sx[v], val, q), J.c, J.c_sh, q);
         } else {
-            J.dst[blk_off<S>(row, xi, step)] = val;
+            p[row_off<TPL>(v, step)] = val;
         }
     }
 }
