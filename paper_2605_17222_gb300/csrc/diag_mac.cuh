@@ -343,6 +343,7 @@ __global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_c
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    pdl_wait();
     __syncthreads();
     volatile u32* abort = &abort_flag;
 
@@ -455,7 +456,7 @@ bool try_ws(const DiagMacArgs& a, cudaStream_t st) {
         attr_set.fetch_or(bit, std::memory_order_release);
     }
     const dim3 grid((N / BLK) * a.batch, a.ext, (a.n3 + K3 - 1) / K3);
-    k_diag_mac_ws<K3, BETA, MINB><<<grid, WS_THREADS, ring + tab, st>>>(a, ring);
+    launch(false, k_diag_mac_ws<K3, BETA, MINB>, grid, WS_THREADS, ring + tab, st, a, ring);
     return true;
 }
 

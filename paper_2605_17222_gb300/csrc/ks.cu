@@ -138,6 +138,7 @@ __global__ void __launch_bounds__(BLK, 8) k_ks_ws(const __grid_constant__ KsArgs
             for (int b = 0; b < BETA; b++) tma_load_1d(st + b * RB, d + b * a.dl.dig, RB, bar);
         }
     };
+    pdl_wait();
     if (l == 0) {
         issue(first);
         if (first + 1 < last) issue(first + 1);
@@ -224,6 +225,7 @@ __global__ void __launch_bounds__(BLK) k_ks_any(const __grid_constant__ KsArgs a
     const bool packed = packed_q(m.q);
     const size_t koff = m.koff + (size_t)run * key_blk(packed, a.beta_max, a.beta_max);
     const size_t o = ((size_t)p.t << a.log_n) + p.s;
+    pdl_wait();
     u64 v0 = 0, v1 = 0;
     if (a.sum) v0 = a.e[0].out0[o], v1 = a.e[0].out1[o];
     for (u32 e = first; e < last; e++) {
@@ -284,6 +286,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_diag_mac(const __grid_constant__
 #pragma unroll
     for (int kk = 0; kk < K3; kk++) acc0[kk] = acc1[kk] = U128{0, 0};
     u32 terms = 0;
+    pdl_wait();
 
     for (u32 j = 0; j < a.n2; j++) {
         const u32 src = j ? auto_src(s, a.gal_mid[j], a.log_n) : s;
@@ -418,7 +421,8 @@ static void run_ks_ws(const KsArgs& a, cudaStream_t st) {
     if (!(done.load(std::memory_order_acquire) & bit) &&
         cudaFuncSetAttribute(k_ks_ws<BETA>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) == cudaSuccess)
         done.fetch_or(bit, std::memory_order_release);
-    k_ks_ws<BETA><<<dim3((1u << a.log_n) / BLK * (a.sum ? 1 : a.count), a.ext), BLK, sm, st>>>(a, stage);
+    const dim3 grid((1u << a.log_n) / BLK * (a.sum ? 1 : a.count), a.ext);
+    launch(false, k_ks_ws<BETA>, grid, BLK, sm, st, a, stage);
 }
 
 void launch_ks(const KsArgs& a, cudaStream_t st) {
@@ -436,7 +440,7 @@ void launch_ks(const KsArgs& a, cudaStream_t st) {
         case 6: run_ks_ws<6>(a, st); break;
         case 7: run_ks_ws<7>(a, st); break;
         case 8: run_ks_ws<8>(a, st); break;
-        default: k_ks_any<<<dim3((1u << a.log_n) / BLK * (a.sum ? 1 : a.count), a.ext), BLK, 0, st>>>(a);
+        default: launch(false, k_ks_any, dim3((1u << a.log_n) / BLK * (a.sum ? 1 : a.count), a.ext), BLK, 0, st, a);
     }
     count_launch();
 }
@@ -475,10 +479,10 @@ void launch_diag_mac(const DiagMacArgs& a, cudaStream_t st) {
         return;
     }
     switch (k3) {
-        case 1: k_diag_mac<1><<<grid, THREADS, 0, st>>>(a); break;
-        case 2: k_diag_mac<2><<<grid, THREADS, 0, st>>>(a); break;
-        case 4: k_diag_mac<4><<<grid, THREADS, 0, st>>>(a); break;
-        default: k_diag_mac<8><<<grid, THREADS, 0, st>>>(a); break;
+        case 1: launch(false, k_diag_mac<1>, grid, THREADS, 0, st, a); break;
+        case 2: launch(false, k_diag_mac<2>, grid, THREADS, 0, st, a); break;
+        case 4: launch(false, k_diag_mac<4>, grid, THREADS, 0, st, a); break;
+        default: launch(false, k_diag_mac<8>, grid, THREADS, 0, st, a); break;
     }
     count_launch();
 }

@@ -139,16 +139,18 @@ ProfScope::~ProfScope() {
 namespace {
 
 // Jobs per launch, passed by value: 510 forward jobs (64 bytes each) and the tables fill the
-// 32,764 bytes of kernel parameters; a level-24 Decompose of three polynomials (504 jobs) is one launch.
-constexpr int MAXJ = 510;
+// 32,764 bytes of kernel parameters; a level-24 Decompose of three polynomials (504 jobs) is one
+// launch.  Launches of up to 60 jobs take a pack of 4 KB: the host copies every byte of the
+// parameters at each launch (1.7 us a launch against 2.7).
+constexpr int MAXJ = 510, SMALLJ = 60;
 static_assert(sizeof(FwdJob) * MAXJ + sizeof(NttTables) <= 32764, "forward jobs exceed the kernel parameter space");
 static_assert(sizeof(InvJob) * MAXJ + sizeof(NttTables) <= 32764, "inverse jobs exceed the kernel parameter space");
 static_assert(sizeof(AddJob) * MAXJ + 64 <= 32764, "add jobs exceed the kernel parameter space");
 constexpr int THREADS = 256;
 
-template <typename J>
+template <typename J, int CAP>
 struct Jobs {
-    J j[MAXJ];
+    J j[CAP];
 };
 
 // Twiddle w and its Shoup companion, one 16-byte load.
@@ -448,9 +450,9 @@ __device__ __forceinline__ void bconv_words(u64* sm, const FwdJob& J, u32 ns, u3
     }
 }
 
-template <int LOGN, int LOGS, bool BCONV>
+template <int LOGN, int LOGS, bool BCONV, int CAP>
 __global__ void __launch_bounds__(THREADS, 4) k_fwd_cols(const __grid_constant__ NttTables T,
-                                                      const __grid_constant__ Jobs<FwdJob> jobs) {
+                                                      const __grid_constant__ Jobs<FwdJob, CAP> jobs) {
     constexpr u32 S = 1u << LOGS, TPL = S / 16, W = THREADS / TPL;
     __shared__ u64 sm[S * W];
     __shared__ __align__(16) ulonglong2 ts[S];
@@ -462,6 +464,10 @@ __global__ void __launch_bounds__(THREADS, 4) k_fwd_cols(const __grid_constant__
     const u64 q = m.q;
     const ulonglong2* tw = T.psi + (size_t)J.mod * N;
     const u32 step = fwd_step(J);
+    // the S - 1 twiddle pairs of the column stages (indices 1 .. S - 1), copied while the words load
+    if (threadIdx.x < S) cp_async16(&ts[threadIdx.x], tw + threadIdx.x);
+    cp_async_commit();
+    pdl_wait();
     if (J.nsrc & FWD_COPY) {  // a pass-through limb: the block copies its columns (every word loaded first)
         u64 y[16];
         if (J.nsrc & FWD_SCALE) {
@@ -477,11 +483,9 @@ __global__ void __launch_bounds__(THREADS, 4) k_fwd_cols(const __grid_constant__
         }
 #pragma unroll
         for (int v = 0; v < 16; v++) J.dst[blk_off<C>(u + TPL * v, col, step)] = y[v];
+        cp_async_wait_all();
         return;
     }
-    // the S - 1 twiddle pairs of the column stages (indices 1 .. S - 1), copied while the words load
-    if (threadIdx.x < S) cp_async16(&ts[threadIdx.x], tw + threadIdx.x);
-    cp_async_commit();
     u64 x[16];
     if constexpr (BCONV) {
         // basis conversion (Eq. 3) of the thread's 16 words, staged through its
@@ -628,9 +632,9 @@ constexpr size_t fwd_rows_smem() {
 }
 
 // Three CTAs per SM (80 registers; measured faster than four at 64).
-template <int LOGN, int LOGS, bool SUBMUL>
+template <int LOGN, int LOGS, bool SUBMUL, int CAP>
 __global__ void __launch_bounds__(THREADS, 3) k_fwd_rows(const __grid_constant__ NttTables T,
-                                                      const __grid_constant__ Jobs<FwdJob> jobs) {
+                                                      const __grid_constant__ Jobs<FwdJob, CAP> jobs) {
     constexpr u32 S = 1u << LOGS, TPL = S / 16, B = THREADS / TPL, SP = S + S / 16;
     constexpr u32 N = 1u << LOGN, log_r = LOGN - LOGS;
     extern __shared__ __align__(16) u64 dsm[];
@@ -639,13 +643,17 @@ __global__ void __launch_bounds__(THREADS, 3) k_fwd_rows(const __grid_constant__
     const u32 u = threadIdx.x % TPL, rl = threadIdx.x / TPL;
     const u32 row = blockIdx.x * B + rl;
     const FwdJob& J = jobs.j[blockIdx.y];
-    if (J.nsrc & FWD_COPY) return;  // copied by the column pass
+    if (J.nsrc & FWD_COPY) {  // copied by the column pass
+        pdl_wait();
+        return;
+    }
     const ModC m = T.mods[J.mod];
     const ulonglong2* tw = T.psi + (size_t)J.mod * N;
     u64* sr = sm + rl * SP;
     ulonglong2* t1 = t1s + rl * T1_STRIDE;
     fwd_rows_stage_twiddles<LOGS>(tw, u, row, log_r, t1);
     cp_async_commit();
+    pdl_wait();
     if (small_q(m.q)) fwd_rows_limb<LOGN, LOGS, SUBMUL, 2>(J, m, tw, sr, t1, u, row);
     else if (m.q < FWD_GROW_MAX) fwd_rows_limb<LOGN, LOGS, SUBMUL, 1>(J, m, tw, sr, t1, u, row);
     else fwd_rows_limb<LOGN, LOGS, SUBMUL, 0>(J, m, tw, sr, t1, u, row);
@@ -693,9 +701,9 @@ __device__ __forceinline__ void inv_rows_stages(u64 (&x)[16], u64* sr, u32 u, u3
     }
 }
 
-template <int LOGN, int LOGS, bool GATHER>
+template <int LOGN, int LOGS, bool GATHER, int CAP>
 __global__ void __launch_bounds__(THREADS, 3) k_inv_rows(const __grid_constant__ NttTables T,
-                                                      const __grid_constant__ Jobs<InvJob> jobs) {
+                                                      const __grid_constant__ Jobs<InvJob, CAP> jobs) {
     constexpr u32 S = 1u << LOGS, TPL = S / 16, B = THREADS / TPL, SP = S + S / 16;
     __shared__ u64 sm[B * SP];
     constexpr u32 N = 1u << LOGN;
@@ -706,6 +714,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_inv_rows(const __grid_constant__
     const ulonglong2* tw = T.ipsi + (size_t)J.mod * N;
     u64* sr = sm + rl * SP;
     const size_t base = (size_t)row * S;
+    pdl_wait();
     u64 x[16];
 #pragma unroll
     for (int v = 0; v < 16; v++) {
@@ -751,9 +760,9 @@ __device__ __forceinline__ void inv_cols_stages(u64 (&x)[16], u64* sm, u32 u, u3
     }
 }
 
-template <int LOGN, int LOGS>
+template <int LOGN, int LOGS, int CAP>
 __global__ void __launch_bounds__(THREADS, 3) k_inv_cols(const __grid_constant__ NttTables T,
-                                                      const __grid_constant__ Jobs<InvJob> jobs) {
+                                                      const __grid_constant__ Jobs<InvJob, CAP> jobs) {
     constexpr u32 S = 1u << LOGS, TPL = S / 16, W = THREADS / TPL;
     __shared__ u64 sm[S * W];
     __shared__ __align__(16) ulonglong2 ts[S];
@@ -766,6 +775,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_inv_cols(const __grid_constant__
     // the S - 1 twiddle pairs of the column stages (indices 1 .. S - 1), copied while the words load
     if (threadIdx.x < S) cp_async16(&ts[threadIdx.x], tw + threadIdx.x);
     cp_async_commit();
+    pdl_wait();
     u64 x[16];
 #pragma unroll
     for (int v = 0; v < 16; v++) x[v] = J.tmp[(size_t)(16 * u + v) * C + col];
@@ -781,34 +791,42 @@ __global__ void k_automorphism(const u64* __restrict__ in, u64* __restrict__ out
     const u32 N = 1u << log_n;
     const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t l = blockIdx.y;
+    pdl_wait();
     if (s < N) out[l * N + s] = in[l * N + auto_src(s, gal, log_n)];
 }
 
-__global__ void k_add_gather(const ModC* __restrict__ mods, const __grid_constant__ Jobs<AddJob> jobs, u32 gal,
+template <int CAP>
+__global__ void k_add_gather(const ModC* __restrict__ mods, const __grid_constant__ Jobs<AddJob, CAP> jobs, u32 gal,
                              int acc, u32 log_n) {
     const u32 N = 1u << log_n;
     const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
     const AddJob& J = jobs.j[blockIdx.y];
     const u64 q = mods[J.mod].q;
+    pdl_wait();
     u64 v = J.a[gal ? auto_src(s, gal, log_n) : s];
     if (J.b) v = add_mod(v, J.b[s], q);
     if (acc) v = add_mod(v, J.out[s], q);
     J.out[s] = v;
 }
 
+template <int CAP, typename J, typename F>
+void with_pack(const J* jobs, int n, F&& f) {
+    Jobs<J, CAP> pack;
+    std::copy(jobs, jobs + n, pack.j);
+    f(pack, n);
+}
 template <typename J, typename F>
 void for_chunks(const J* jobs, int njobs, F&& f) {
     for (int s = 0; s < njobs; s += MAXJ) {
-        Jobs<J> pack;
         const int n = std::min(MAXJ, njobs - s);
-        for (int i = 0; i < n; i++) pack.j[i] = jobs[s + i];
-        f(pack, n);
+        if (n <= SMALLJ) with_pack<SMALLJ>(jobs + s, n, f);
+        else with_pack<MAXJ>(jobs + s, n, f);
     }
 }
 
-template <int LR, int LC>
-void fwd_impl(const NttTables& T, const Jobs<FwdJob>& p, int n, bool bconv, bool submul, cudaStream_t st) {
+template <int LR, int LC, int CAP>
+void fwd_impl(const NttTables& T, const Jobs<FwdJob, CAP>& p, int n, bool bconv, bool submul, cudaStream_t st) {
     const u32 N = 1u << T.log_n;
     const dim3 g1((N >> LR) / (THREADS / ((1u << LR) / 16)), n), g2((N >> LC) / (THREADS / ((1u << LC) / 16)), n);
     int nt = 0;  // transformed limbs (copy jobs aside)
@@ -820,8 +838,8 @@ void fwd_impl(const NttTables& T, const Jobs<FwdJob>& p, int n, bool bconv, bool
             if (!(p.j[i].nsrc & FWD_COPY)) bconv_macs += (double)(p.j[i].nsrc & 0xFFFFu) * N;
     {
         ProfScope ps(K_FWD_COLS, st, bconv_macs, half * LR);
-        if (bconv) k_fwd_cols<LR + LC, LR, true><<<g1, THREADS, 0, st>>>(T, p);
-        else k_fwd_cols<LR + LC, LR, false><<<g1, THREADS, 0, st>>>(T, p);
+        if (bconv) launch(false, k_fwd_cols<LR + LC, LR, true, CAP>, g1, THREADS, 0, st, T, p);
+        else launch(false, k_fwd_cols<LR + LC, LR, false, CAP>, g1, THREADS, 0, st, T, p);
     }
     {
         if (!nt) return;  // copies only
@@ -829,28 +847,29 @@ void fwd_impl(const NttTables& T, const Jobs<FwdJob>& p, int n, bool bconv, bool
         constexpr size_t sm = fwd_rows_smem<LC>();
         static std::atomic<uint64_t> lim_t{0}, lim_f{0};
         if (submul) {
-            smem_limit(k_fwd_rows<LR + LC, LC, true>, sm, lim_t);
-            k_fwd_rows<LR + LC, LC, true><<<g2, THREADS, sm, st>>>(T, p);
+            smem_limit(k_fwd_rows<LR + LC, LC, true, CAP>, sm, lim_t);
+            launch(true, k_fwd_rows<LR + LC, LC, true, CAP>, g2, THREADS, sm, st, T, p);
         } else {
-            smem_limit(k_fwd_rows<LR + LC, LC, false>, sm, lim_f);
-            k_fwd_rows<LR + LC, LC, false><<<g2, THREADS, sm, st>>>(T, p);
+            smem_limit(k_fwd_rows<LR + LC, LC, false, CAP>, sm, lim_f);
+            launch(true, k_fwd_rows<LR + LC, LC, false, CAP>, g2, THREADS, sm, st, T, p);
         }
     }
 }
 
-template <int LR, int LC>
-void inv_impl(const NttTables& T, const Jobs<InvJob>& p, int n, bool gather, cudaStream_t st) {
+template <int LR, int LC, int CAP>
+void inv_impl(const NttTables& T, const Jobs<InvJob, CAP>& p, int n, bool gather, cudaStream_t st) {
     const u32 N = 1u << T.log_n;
     const dim3 g1((N >> LR) / (THREADS / ((1u << LR) / 16)), n), g2((N >> LC) / (THREADS / ((1u << LC) / 16)), n);
     const double half = (double)n * (N / 2);
+    const bool early = g2.x * g2.y < 64;
     {
         ProfScope ps(K_INV_ROWS, st, 0, half * LC);
-        if (gather) k_inv_rows<LR + LC, LC, true><<<g2, THREADS, 0, st>>>(T, p);
-        else k_inv_rows<LR + LC, LC, false><<<g2, THREADS, 0, st>>>(T, p);
+        if (gather) launch(early, k_inv_rows<LR + LC, LC, true, CAP>, g2, THREADS, 0, st, T, p);
+        else launch(early, k_inv_rows<LR + LC, LC, false, CAP>, g2, THREADS, 0, st, T, p);
     }
     {
         ProfScope ps(K_INV_COLS, st, 0, half * LR);
-        k_inv_cols<LR + LC, LR><<<g1, THREADS, 0, st>>>(T, p);
+        launch(true, k_inv_cols<LR + LC, LR, CAP>, g1, THREADS, 0, st, T, p);
     }
 }
 
@@ -929,7 +948,7 @@ void launch_fwd_ntt(const NttTables& T, const FwdJob* jobs, int njobs, cudaStrea
             submul = jobs[i].subout != nullptr;
             break;
         }
-    for_chunks(jobs, njobs, [&](const Jobs<FwdJob>& p, int n) {
+    for_chunks(jobs, njobs, [&](const auto& p, int n) {
         NTT_DISPATCH(fwd_impl, bconv, submul);
         count_launch(transforms ? 2 : 1);
     });
@@ -938,7 +957,7 @@ void launch_fwd_ntt(const NttTables& T, const FwdJob* jobs, int njobs, cudaStrea
 void launch_inv_ntt(const NttTables& T, const InvJob* jobs, int njobs, cudaStream_t st) {
     if (njobs <= 0) return;
     const bool gather = jobs[0].gal != 0;
-    for_chunks(jobs, njobs, [&](const Jobs<InvJob>& p, int n) {
+    for_chunks(jobs, njobs, [&](const auto& p, int n) {
         NTT_DISPATCH(inv_impl, gather);
         count_launch(2);
     });
@@ -948,7 +967,7 @@ void launch_automorphism(const u64* in, u64* out, u32 n_limbs, u32 gal, u32 log_
     if (!n_limbs) return;
     const u32 N = 1u << log_n;
     ProfScope ps(K_AUTO, st);
-    k_automorphism<<<dim3((N + 255) / 256, n_limbs), 256, 0, st>>>(in, out, gal, log_n);
+    launch(true, k_automorphism, dim3((N + 255) / 256, n_limbs), 256, 0, st, in, out, gal, log_n);
     count_launch();
 }
 
@@ -1009,9 +1028,10 @@ cudaError_t probe_int_rates(u32 blocks, double* macs_per_s, double* butterflies_
 void launch_add_gather(const ModC* mods, const AddJob* jobs, int njobs, u32 gal, int accumulate, u32 log_n,
                        cudaStream_t st) {
     const u32 N = 1u << log_n;
-    for_chunks(jobs, njobs, [&](const Jobs<AddJob>& p, int n) {
+    for_chunks(jobs, njobs, [&](const auto& p, int n) {
         ProfScope ps(K_ADD, st);
-        k_add_gather<<<dim3((N + 255) / 256, n), 256, 0, st>>>(mods, p, gal, accumulate, log_n);
+        launch(true, k_add_gather<std::extent<decltype(p.j)>::value>, dim3((N + 255) / 256, n), 256, 0, st, mods, p, gal,
+                   accumulate, log_n);
         count_launch();
     });
 }
