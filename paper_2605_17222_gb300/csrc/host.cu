@@ -125,6 +125,8 @@ struct LevelConsts {
     // ModDown: per P limb, N^-1 (P/p_i)^-1; table [level][k] of [P/p_i]_{q_j}; P^-1 mod q_j
     std::vector<u64> md_c, md_sh, md_pinv, md_pinv_sh;
     u64* md_tab = nullptr;
+    // ModDown into Decompose: per Q limb j, P^-1 dec_c mod q_j and N times it
+    std::vector<u64> mdd_c, mdd_sh, mdd_c2, mdd_c2_sh;
     // ModDown+rescale over {q_{l-1}, p_0..}: same shapes with k+1 sources, level-1 targets
     std::vector<u64> mdr_c, mdr_sh, mdr_pinv, mdr_pinv_sh;
     u64* mdr_tab = nullptr;
@@ -309,6 +311,13 @@ const LevelConsts& ckks_ctx::lc(u32 level) {
     std::vector<u32> P;
     for (u32 i = 0; i < K; i++) P.push_back(L + i);
     down(P, level, c.md_c, c.md_sh, c.md_pinv, c.md_pinv_sh, c.md_tab);
+    for (u32 j = 0; j < level; j++) {
+        const u64 q = mods[j], v = mulmod_h(c.dec_c[j], c.md_pinv[j], q), w = mulmod_h(v, N % q, q);
+        c.mdd_c.push_back(v);
+        c.mdd_sh.push_back(shoup_h(v, q));
+        c.mdd_c2.push_back(w);
+        c.mdd_c2_sh.push_back(shoup_h(w, q));
+    }
     if (level >= 2) {
         std::vector<u32> S{level - 1};
         for (u32 i = 0; i < K; i++) S.push_back(L + i);
@@ -358,20 +367,43 @@ void release_lanes(ckks_ctx* C, cudaStream_t st) {
 }
 
 // ------------------------------------------------------------------ key switching steps
+// The forward jobs of a Decompose of one polynomial: for each digit, basis
+// conversions of its limbs in Y [level][N] to the limbs outside it.
+void digit_jobs(const ckks_ctx* C, const LevelConsts& LC, u32 level, u64* Y, u64* digits, const DigLayout& dl, u32 step,
+                std::vector<FwdJob>& fj) {
+    const u32 N = C->N, ext = level + C->K, beta = C->beta(level);
+    for (u32 b = 0; b < beta; b++) {
+        const u32 first = b * C->alpha, n = std::min(C->alpha, level - first);
+        // the digit's words are canonical residues of its moduli: below 2^40 if every one is
+        bool small = true;
+        for (u32 j = first; j < first + n; j++) small = small && C->mods[j] < (1ull << 40);
+        for (u32 t = 0; t < ext; t++) {
+            if (t >= first && t < first + n) continue;
+            fj.push_back(FwdJob{Y + (size_t)first * N, digits + b * dl.dig + t * dl.limb,
+                                LC.dec_tab + ((size_t)b * ext + t) * C->alpha, nullptr, 0, 0, C->gmod(level, t),
+                                n | (small ? 1u << 16 : 0u) | step});
+        }
+    }
+}
+
+DigLayout digit_layout(const ckks_ctx* C, u32 level, u32 slots) {
+    return slots ? grouped_digits(slots, C->log_n) : plain_digits(level + C->K, C->log_n);
+}
+
 // Decompose (Fig. 1, Eq. 3) of `count` polynomials at once: c_i [level][N]
-// (gathered through x -> x^gal if gal) -> digits_i [beta][level+K][N].
-// Y: scratch [count][level][N].  One launch pair per transform direction
-// covers every polynomial, so small steps still fill the GPU.
+// (gathered through x -> x^gals[i]; none if gals is empty) -> digits_i
+// [beta][level+K][N].  Y: scratch [count][level][N].  One launch pair per
+// transform direction covers every polynomial, so small steps still fill the GPU.
 // slots: 0 for plain digits, else the slots of grouped digits (DigLayout), of
 // which the digits take the first beta.
 // extra: further elementwise jobs (FWD_COPY) to run in the forward launch.
-void op_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& cs, u32 gal,
+void op_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& cs, const std::vector<u32>& gals,
                         const std::vector<u64*>& digits, u32 slots, u64* Y, cudaStream_t st,
                         const std::vector<FwdJob>* extra = nullptr) {
     const LevelConsts& LC = C->lc(level);
-    const u32 N = C->N, ext = level + C->K, beta = C->beta(level);
+    const u32 N = C->N, beta = C->beta(level);
     const u32 cnt = (u32)cs.size();
-    const DigLayout dl = slots ? grouped_digits(slots, C->log_n) : plain_digits(ext, C->log_n);
+    const DigLayout dl = digit_layout(C, level, slots);
     const u32 step = slots << FWD_STEP;
     std::vector<InvJob> ij;
     ij.reserve((size_t)cnt * level);
@@ -379,31 +411,19 @@ void op_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& c
         u64* Yp = Y + (size_t)p * level * N;
         for (u32 j = 0; j < level; j++)
             ij.push_back(InvJob{cs[p] + (size_t)j * N, Yp + (size_t)j * N, Yp + (size_t)j * N, LC.dec_c[j], LC.dec_sh[j],
-                                j, gal});
+                                j, gals.empty() ? 0 : gals[p]});
     }
     launch_inv_ntt(C->T, ij.data(), (int)ij.size(), st);
     std::vector<FwdJob> fj;
     for (u32 p = 0; p < cnt; p++) {
-        u64* Yp = Y + (size_t)p * level * N;
-        for (u32 b = 0; b < beta; b++) {
-            const u32 first = b * C->alpha, n = std::min(C->alpha, level - first);
-            // the digit's words are canonical residues of its moduli: below 2^40 if every one is
-            bool small = true;
-            for (u32 j = first; j < first + n; j++) small = small && C->mods[j] < (1ull << 40);
-            for (u32 t = 0; t < ext; t++) {
-                if (t >= first && t < first + n) continue;
-                fj.push_back(FwdJob{Yp + (size_t)first * N, digits[p] + b * dl.dig + t * dl.limb,
-                                    LC.dec_tab + ((size_t)b * ext + t) * C->alpha, nullptr, nullptr, 0, 0,
-                                    C->gmod(level, t), n | (small ? 1u << 16 : 0u) | step});
-            }
-        }
+        digit_jobs(C, LC, level, Y + (size_t)p * level * N, digits[p], dl, step, fj);
         // each digit's own limbs are the (gathered) input limbs: copy jobs in the same launch, after
         // the polynomial's transforms, so that they fill the transforms' last wave
         for (u32 b = 0; b < beta; b++) {
             const u32 first = b * C->alpha, n = std::min(C->alpha, level - first);
             for (u32 j = first; j < first + n; j++)
                 fj.push_back(FwdJob{cs[p] + (size_t)j * N, digits[p] + b * dl.dig + j * dl.limb, nullptr, nullptr,
-                                    nullptr, gal, 0, j, FWD_COPY | step});
+                                    gals.empty() ? 0 : gals[p], 0, j, FWD_COPY | step});
         }
     }
     if (extra) fj.insert(fj.end(), extra->begin(), extra->end());
@@ -411,14 +431,14 @@ void op_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& c
 }
 
 void op_decompose(ckks_ctx* C, u32 level, const u64* c, u32 gal, u64* digits, u64* Y, cudaStream_t st) {
-    op_decompose_batch(C, level, std::vector<const u64*>{c}, gal, std::vector<u64*>{digits}, 0, Y, st);
+    op_decompose_batch(C, level, {c}, std::vector<u32>(gal ? 1 : 0, gal), {digits}, 0, Y, st);
 }
 
 // P c0 (Alg. 2 line 2) as scaling jobs: the Q limbs of a plain c0 to dst, whose
 // limbs lie `limb` words apart and their blocks `slots` blocks apart.
 void lift_jobs(const ckks_ctx* C, u32 level, const u64* c0, u64* dst, u64 limb, u32 slots, std::vector<FwdJob>& out) {
     for (u32 t = 0; t < level; t++)
-        out.push_back(FwdJob{c0 + (size_t)t * C->N, dst + t * limb, nullptr, nullptr, nullptr, C->lift_c[t],
+        out.push_back(FwdJob{c0 + (size_t)t * C->N, dst + t * limb, nullptr, nullptr, C->lift_c[t],
                              C->lift_sh[t], t, FWD_COPY | FWD_SCALE | slots << FWD_STEP});
 }
 
@@ -442,7 +462,7 @@ void op_down_batch(ckks_ctx* C, const std::vector<const u64*>& xs, u32 src_first
     for (u32 p = 0; p < cnt; p++)
         for (u32 j = 0; j < ntgt; j++)
             fj.push_back(FwdJob{Y + (size_t)p * ns * N, outs[p] + (size_t)j * N, tab + (size_t)j * ns,
-                                xs[p] + (size_t)j * N, outs[p] + (size_t)j * N, inv[j], inv_sh[j], j, ns});
+                                xs[p] + (size_t)j * N, inv[j], inv_sh[j], j, ns});
     launch_fwd_ntt(C->T, fj.data(), (int)fj.size(), st);
 }
 
@@ -452,6 +472,67 @@ void op_moddown_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& xs,
     std::vector<u32> g;
     for (u32 i = 0; i < C->K; i++) g.push_back(C->L + i);
     op_down_batch(C, xs, level, g, LC.md_c, LC.md_sh, LC.md_tab, level, LC.md_pinv, LC.md_pinv_sh, outs, Y, st);
+}
+
+// Decompose(ModDown(x_i)) of extended polynomials (Alg. 2 lines 6-7 and
+// 15-16), the digits as from op_decompose_batch.  The ModDown's output is
+// needed in both domains: its coefficients for the basis conversions, as
+// INTT(x) minus the conversion of the special limbs (launch_inv_conv), and its
+// NTT words for the digits' own limbs, as the ModDown tail of forward jobs that
+// join the conversions' launch and write the digits in place.  Five launches
+// and no ModDown polynomial in memory, where the two steps one after the other
+// are eight and write it, read it back and copy it (N = 2^16 level 9, (2,8,4):
+// 688 -> 670 us).  The price is the special limbs' conversion a second time,
+// K products a word, so it pays where launches count: up to 3 * 2^20 words of
+// Q limbs (N = 2^16 level 24, three polynomials, 4.5 * 2^20: 2.818 ms fused, 2.810
+// not; N = 2^15 level 11, 2.3 * 2^20: 574 and 577 us), or 2^20 with more than
+// four special limbs (Set-B, K = 8, 2^21.6: 1.45 and 1.435 ms; Set-A, K = 5,
+// 2^19.2: 1.367 and 1.381 ms).
+// Y: scratch [count][K + level][N].
+void op_moddown_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& xs,
+                                const std::vector<u64*>& digits, u32 slots, u64* Y, cudaStream_t st) {
+    const LevelConsts& LC = C->lc(level);
+    const u32 N = C->N, K = C->K, cnt = (u32)xs.size();
+    if ((u64)cnt * level * N > (K > 4 ? 1u << 20 : 3u << 20)) {
+        Arena ar(st, N);
+        std::vector<u64*> tq;
+        for (u32 p = 0; p < cnt; p++) tq.push_back(ar.limbs(level));
+        op_moddown_batch(C, level, xs, tq, Y, st);
+        op_decompose_batch(C, level, {tq.begin(), tq.end()}, {}, digits, slots, Y, st);
+        return;
+    }
+    const DigLayout dl = digit_layout(C, level, slots);
+    const u32 step = slots << FWD_STEP;
+    std::vector<InvJob> pj;
+    std::vector<InvConvJob> qj;
+    std::vector<FwdJob> fj;
+    for (u32 p = 0; p < cnt; p++) {
+        u64 *YP = Y + (size_t)p * (K + level) * N, *YQ = YP + (size_t)K * N;
+        for (u32 i = 0; i < K; i++)
+            pj.push_back(InvJob{xs[p] + (size_t)(level + i) * N, YP + (size_t)i * N, YP + (size_t)i * N, LC.md_c[i],
+                                LC.md_sh[i], C->L + i, 0});
+        for (u32 j = 0; j < level; j++) {
+            InvConvJob q;
+            static_cast<InvJob&>(q) = InvJob{xs[p] + (size_t)j * N, YQ + (size_t)j * N, YQ + (size_t)j * N, LC.mdd_c[j],
+                                             LC.mdd_sh[j], j, 0};
+            q.csrc = YP;
+            q.bcst = LC.md_tab + (size_t)j * K;
+            q.c2 = LC.mdd_c2[j];
+            q.c2_sh = LC.mdd_c2_sh[j];
+            q.nsrc = K;
+            q.pad = 0;
+            qj.push_back(q);
+        }
+        digit_jobs(C, LC, level, YQ, digits[p], dl, step, fj);
+    }
+    for (u32 p = 0; p < cnt; p++) {
+        const u64* YP = Y + (size_t)p * (K + level) * N;
+        for (u32 j = 0; j < level; j++)
+            fj.push_back(FwdJob{YP, digits[p] + j / C->alpha * dl.dig + j * dl.limb, LC.md_tab + (size_t)j * K,
+                                xs[p] + (size_t)j * N, LC.md_pinv[j], LC.md_pinv_sh[j], j, K | step});
+    }
+    launch_inv_conv(C->T, pj.data(), (int)pj.size(), qj.data(), (int)qj.size(), st);
+    launch_fwd_ntt(C->T, fj.data(), (int)fj.size(), st);
 }
 
 void op_moddown(ckks_ctx* C, u32 level, const u64* x, u64* out, u64* Y, cudaStream_t st) {
@@ -528,15 +609,6 @@ void op_ks_list(KsArgs& a, const std::vector<KsItem>& items, cudaStream_t st) {
     }
 }
 
-void op_add_gather(ckks_ctx* C, u32 nlimbs, u32 level, const u64* a, const u64* b, u64* out, u32 gal, int acc,
-                   cudaStream_t st) {
-    std::vector<AddJob> j(nlimbs);
-    for (u32 t = 0; t < nlimbs; t++)
-        j[t] = AddJob{a + (size_t)t * C->N, b ? b + (size_t)t * C->N : nullptr, out + (size_t)t * C->N,
-                      C->gmod(level, t), 0};
-    launch_add_gather((const ModC*)C->d_mods.p, j.data(), (int)nlimbs, gal, acc, C->log_n, st);
-}
-
 // tile: the diagonal kernel's outer indices per CTA (0 = default; see DiagMacArgs).
 DiagMacArgs dm_base(ckks_ctx* C, u32 level, bool with_p, const ckks_diags* f, u32 tile = 0) {
     DiagMacArgs a;
@@ -606,7 +678,7 @@ void sched_th(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 
     const int64_t s = f->stride;
     Arena ar(st, N);
     const u32 nb = std::max<u32>(1, std::max(n1 - 1, n3));  // widest batch of the key-switch phases
-    u64* Y = ar.limbs(std::max<size_t>((size_t)nb * level, 2 * (C->K + 1)));
+    u64* Y = ar.limbs((size_t)nb * ext + C->K + 2);
     const bool mid = n2 > 1;
     const u32 slots = mid ? beta + 1 : 1;  // of X_i: its digits and A_i, or A_i alone
     std::vector<u64*> X(n1, nullptr), B(n1, nullptr);
@@ -616,7 +688,7 @@ void sched_th(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 
     // P c0 (line 2) into X_0's last slot: scaling jobs of the line-1 Decompose's forward launch
     std::vector<FwdJob> lift;
     lift_jobs(C, level, io.c0, X[0] + (size_t)(slots - 1) * BLK, (u64)slots * N, slots, lift);
-    if (D0) op_decompose_batch(C, level, {io.c1}, 0, {D0}, d_slots, Y, st, &lift);  // line 1
+    if (D0) op_decompose_batch(C, level, {io.c1}, {}, {D0}, d_slots, Y, st, &lift);  // line 1
     else launch_fwd_ntt(C->T, lift.data(), (int)lift.size(), st);  // no rotation but the outer ones
     if (n1 > 1) {  // lines 2-5 for every i at once (the lift is fused)
         std::vector<KsItem> es;
@@ -629,16 +701,7 @@ void sched_th(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 
         op_ks_list(k, es, st);
     }
     if (mid && n1 > 1) {  // lines 6-7 for every i at once
-        std::vector<const u64*> bs, tqc;
-        std::vector<u64*> tq, dg;
-        for (u32 i = 1; i < n1; i++) {
-            bs.push_back(B[i]);
-            tq.push_back(ar.limbs(level));
-            tqc.push_back(tq.back());
-            dg.push_back(X[i]);
-        }
-        op_moddown_batch(C, level, bs, tq, Y, st);
-        op_decompose_batch(C, level, tqc, 0, dg, slots, Y, st);
+        op_moddown_decompose_batch(C, level, {B.begin() + 1, B.end()}, {X.begin() + 1, X.end()}, slots, Y, st);
     }
     DiagMacArgs a = dm_base(C, level, true, f, tile);
     a.n1 = n1;
@@ -670,16 +733,13 @@ void sched_th(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 
         CK(cudaMemsetAsync(acc1, 0, (size_t)ext * N * sizeof(u64), st));
     }
     if (!ol.rotated.empty()) {  // lines 15-18 for every rotated k at once
-        std::vector<const u64*> us, tqc;
-        std::vector<u64*> tq, dk;
+        std::vector<const u64*> us;
+        std::vector<u64*> dk;
         for (u32 k : ol.rotated) {
             us.push_back(U1[k]);
-            tq.push_back(ar.limbs(level));
-            tqc.push_back(tq.back());
             dk.push_back(ar.limbs((size_t)beta * ext));
         }
-        op_moddown_batch(C, level, us, tq, Y, st);
-        op_decompose_batch(C, level, tqc, 0, dk, beta, Y, st);
+        op_moddown_decompose_batch(C, level, us, dk, beta, Y, st);
         std::vector<KsItem> es;
         for (size_t c = 0; c < ol.rotated.size(); c++) {
             const u32 k = ol.rotated[c];
@@ -709,7 +769,7 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
     const int64_t s = f->stride;
     Arena ar(st, N);
     const u32 nb = std::max<u32>(1, std::max(n1 - 1, n3)) * nbat;
-    u64* Y = ar.limbs(std::max<size_t>((size_t)std::max(nb, nbat) * level, 2ull * nbat * (C->K + 1)));
+    u64* Y = ar.limbs((size_t)nb * ext + (size_t)nbat * (C->K + 2));
     const bool mid = n2 > 1;
     const u32 slots = mid ? beta + 1 : 1;  // of X_i: its digits and A_i, or A_i alone
     u64* Xall = ar.limbs((size_t)nbat * n1 * slots * ext);  // [b][i][ext][N/BLK][slots][BLK]
@@ -731,7 +791,7 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
             cs.push_back(ios[b].c1);
             ds.push_back(Dp(b));
         }
-        if (mid || n1 > 1) op_decompose_batch(C, level, cs, 0, ds, d_slots, Y, st, &lift);
+        if (mid || n1 > 1) op_decompose_batch(C, level, cs, {}, ds, d_slots, Y, st, &lift);
         else launch_fwd_ntt(C->T, lift.data(), (int)lift.size(), st);
     }
     if (n1 > 1) {  // lines 2-5, every (i, b) in launches of KS_MAX products
@@ -746,17 +806,14 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
         op_ks_list(k, es, st);
     }
     if (mid && n1 > 1) {  // lines 6-7
-        std::vector<const u64*> bs, tqc;
-        std::vector<u64*> tq, dg;
+        std::vector<const u64*> bs;
+        std::vector<u64*> dg;
         for (u32 b = 0; b < nbat; b++)
             for (u32 i = 1; i < n1; i++) {
                 bs.push_back(Bp(b, i));
-                tq.push_back(ar.limbs(level));
-                tqc.push_back(tq.back());
                 dg.push_back(Xp(b, i));
             }
-        op_moddown_batch(C, level, bs, tq, Y, st);
-        op_decompose_batch(C, level, tqc, 0, dg, slots, Y, st);
+        op_moddown_decompose_batch(C, level, bs, dg, slots, Y, st);
     }
     DiagMacArgs a = dm_base(C, level, true, f, tile);
     a.n1 = n1;
@@ -792,17 +849,14 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
     };
     const size_t nrot = ol.rotated.size();
     if (nrot) {  // lines 15-18
-        std::vector<const u64*> us, tqc;
-        std::vector<u64*> tq, dk;
+        std::vector<const u64*> us;
+        std::vector<u64*> dk;
         for (u32 b = 0; b < nbat; b++)
             for (u32 k : ol.rotated) {
                 us.push_back(Up(b, k, 1));
-                tq.push_back(ar.limbs(level));
-                tqc.push_back(tq.back());
                 dk.push_back(ar.limbs(dig));
             }
-        op_moddown_batch(C, level, us, tq, Y, st);
-        op_decompose_batch(C, level, tqc, 0, dk, beta, Y, st);
+        op_moddown_decompose_batch(C, level, us, dk, beta, Y, st);
         for (u32 b = 0; b < nbat; b++) {
             std::vector<KsItem> es;
             for (size_t c = 0; c < nrot; c++) {
@@ -829,28 +883,50 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
 
 // BSGS, Eq. (5): un-hoisted rotations (each with its own Decompose of the
 // rotated c1 and two ModDowns), products over Q, plain rescale at the end.
-void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 n2, cudaStream_t st,
-                u32 tile = 0) {
-    const u32 N = C->N, ext = level + C->K, beta = C->beta(level);
+// The baby steps are independent of one another, and so are the giant steps:
+// each layer runs in chunks of rotations, every step of a chunk one launch.
+void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 n2, cudaStream_t st, u32 tile = 0) {
+    const u32 N = C->N, K = C->K, ext = level + K, beta = C->beta(level);
     const int64_t s = f->stride;
     Arena ar(st, N);
-    u64* Y = ar.limbs(std::max(level, C->K + 1));
-    u64* D = ar.limbs((size_t)beta * ext);
-    u64* X0 = ar.limbs(ext);
-    u64* X1 = ar.limbs(ext);
-    u64* T0 = ar.limbs(level);
-    auto rotate_into = [&](const u64* c0, const u64* c1, int64_t r, u64* o0, u64* o1, int acc) {
-        const u32 g = C->galois(r);
-        op_decompose(C, level, c1, g, D, Y, st);
-        op_ks_inner(C, level, D, key_of(C, r), 0, nullptr, 0, X0, X1, 0, st);
-        op_moddown(C, level, X0, T0, Y, st);
-        if (acc) {
-            op_add_gather(C, level, level, c0, T0, o0, g, 1, st);
-            op_moddown(C, level, X1, X0, Y, st);  // reuse X0 as [level] scratch
-            op_add_gather(C, level, level, X0, nullptr, o1, 0, 1, st);
-        } else {
-            op_add_gather(C, level, level, c0, T0, o0, g, 0, st);
-            op_moddown(C, level, X1, o1, Y, st);
+    const OuterLayer ol = outer_layer(C, f, n1, n2);
+    struct Rot {
+        const u64 *c0, *c1;
+        int64_t r;
+        u64 *o0, *o1;  // T0 = ModDown of the first output and the rotated second component
+    };
+    // limbs of scratch per rotation: digits, the two products, ModDown and Decompose sources; a
+    // chunk takes at most 512 MB of it (one rotation at least)
+    const size_t per = (size_t)beta * ext + 2 * ext + std::max<size_t>(level, 2 * K);
+    const u32 widest = std::max<u32>(1, std::max<u32>(n1 - 1, (u32)ol.rotated.size()));
+    const u32 chunk = (u32)std::min<size_t>(widest, std::max<size_t>(1, (size_t(512) << 20) / (per * N * 8)));
+    u64* D = ar.limbs((size_t)chunk * beta * ext);
+    u64* P = ar.limbs((size_t)chunk * 2 * ext);
+    u64* Y = ar.limbs(std::max<size_t>((size_t)chunk * std::max(level, 2 * K), 4));
+    // ModDown(<Decompose(phi_r(c1)), swk_r>) of every rotation into (o0, o1)
+    auto switch_keys = [&](const std::vector<Rot>& rots) {
+        for (size_t b = 0; b < rots.size(); b += chunk) {
+            const u32 n = (u32)std::min<size_t>(chunk, rots.size() - b);
+            std::vector<const u64*> cs, xs;
+            std::vector<u32> gals;
+            std::vector<u64*> ds, outs;
+            std::vector<KsItem> es;
+            for (u32 i = 0; i < n; i++) {
+                const Rot& R = rots[b + i];
+                cs.push_back(R.c1);
+                gals.push_back(C->galois(R.r));
+                ds.push_back(D + (size_t)i * beta * ext * N);
+                u64 *x0 = P + (size_t)i * 2 * ext * N, *x1 = x0 + (size_t)ext * N;
+                es.push_back(KsItem{ds[i], key_of(C, R.r), nullptr, x0, x1, 0, 0});
+                xs.push_back(x0);
+                xs.push_back(x1);
+                outs.push_back(R.o0);
+                outs.push_back(R.o1);
+            }
+            op_decompose_batch(C, level, cs, gals, ds, beta, Y, st);
+            KsArgs k = ks_base(C, level, beta, 0);
+            op_ks_list(k, es, st);
+            op_moddown_batch(C, level, xs, outs, Y, st);
         }
     };
     DiagMacArgs a = dm_base(C, level, false, f, tile);
@@ -860,14 +936,20 @@ void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u3
     a.slots = 1;
     a.X[0] = io.c0;
     a.B[0] = io.c1;
-    for (u32 i = 1; i < n1; i++) {
-        u64* c0 = ar.limbs(level);
-        u64* c1 = ar.limbs(level);
-        rotate_into(io.c0, io.c1, s * i, c0, c1, 0);
-        a.X[i] = c0;
-        a.B[i] = c1;
+    if (n1 > 1) {
+        std::vector<Rot> rots;
+        std::vector<AddJob> add;
+        for (u32 i = 1; i < n1; i++) {
+            u64 *t0 = ar.limbs(level), *c0 = ar.limbs(level), *c1 = ar.limbs(level);
+            rots.push_back(Rot{io.c0, io.c1, s * i, t0, c1});
+            a.X[i] = c0;
+            a.B[i] = c1;
+            for (u32 t = 0; t < level; t++)
+                add.push_back(AddJob{io.c0 + (size_t)t * N, t0 + (size_t)t * N, c0 + (size_t)t * N, t, C->galois(s * i)});
+        }
+        switch_keys(rots);
+        launch_add_gather((const ModC*)C->d_mods.p, add.data(), (int)add.size(), C->log_n, st);
     }
-    const OuterLayer ol = outer_layer(C, f, n1, n2);
     std::vector<u64*> V0(n2), V1(n2);
     for (u32 j = 0; j < n2; j++) {
         V0[j] = ar.limbs(level);
@@ -883,9 +965,30 @@ void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u3
         CK(cudaMemsetAsync(acc0, 0, (size_t)level * N * sizeof(u64), st));
         CK(cudaMemsetAsync(acc1, 0, (size_t)level * N * sizeof(u64), st));
     }
-    for (u32 j : ol.rotated) rotate_into(V0[j], V1[j], ol.amount[j], acc0, acc1, 1);
-    op_rescale(C, level, acc0, io.o0, Y, st);
-    op_rescale(C, level, acc1, io.o1, Y, st);
+    if (!ol.rotated.empty()) {
+        std::vector<Rot> rots;
+        for (u32 j : ol.rotated) rots.push_back(Rot{V0[j], V1[j], ol.amount[j], ar.limbs(level), ar.limbs(level)});
+        switch_keys(rots);
+        for (size_t b = 0; b < rots.size(); b += SUM_MAX) {
+            SumArgs m;
+            memset(&m, 0, sizeof(m));
+            m.count = (u32)std::min<size_t>(SUM_MAX, rots.size() - b);
+            for (u32 k = 0; k < m.count; k++) {
+                const Rot& R = rots[b + k];
+                m.a[k] = R.c0;
+                m.b0[k] = R.o0;
+                m.b1[k] = R.o1;
+                m.gal[k] = C->galois(R.r);
+            }
+            m.acc0 = acc0;
+            m.acc1 = acc1;
+            m.mods = (const ModC*)C->d_mods.p;
+            m.level = level;
+            m.log_n = C->log_n;
+            launch_sum_gather(m, st);
+        }
+    }
+    op_rescale_batch(C, level, {acc0, acc1}, {io.o0, io.o1}, Y, st);
 }
 
 void validate_split(lt_algo algo, u32 D, const lt_split& sp) {
@@ -2105,7 +2208,7 @@ ckks_status ckks_poly_ntt(ckks_ctx* ctx, uint64_t* poly, uint32_t level, int ext
         } else {
             std::vector<FwdJob> j(nl);
             for (u32 t = 0; t < nl; t++)
-                j[t] = FwdJob{poly + (size_t)t * N, poly + (size_t)t * N, nullptr, nullptr, nullptr, 0, 0,
+                j[t] = FwdJob{poly + (size_t)t * N, poly + (size_t)t * N, nullptr, nullptr, 0, 0,
                               ctx->gmod(level, t), 0};
             launch_fwd_ntt(ctx->T, j.data(), (int)nl, (cudaStream_t)stream);
         }
@@ -2218,7 +2321,7 @@ ckks_status ckks_moddown_noalloc(ckks_ctx* ctx, uint32_t level, const uint64_t* 
         launch_inv_ntt(ctx->T, ij, (int)k, st);
         FwdJob fj[64];
         for (u32 j = 0; j < level; j++)
-            fj[j] = FwdJob{Y, out + (size_t)j * N, LC->md_tab + (size_t)j * k, x + (size_t)j * N, out + (size_t)j * N,
+            fj[j] = FwdJob{Y, out + (size_t)j * N, LC->md_tab + (size_t)j * k, x + (size_t)j * N,
                            LC->md_pinv[j], LC->md_pinv_sh[j], j, k};
         launch_fwd_ntt(ctx->T, fj, (int)level, st);
         CK(cudaGetLastError());

@@ -22,6 +22,7 @@ namespace ckks {
 // in small grids (1.70 -> 1.61); the forward column pass, the key products and
 // the diagonal kernel not, whose early CTAs only share SMs with the kernel
 // before (everything early: Set-A 1.48 ms against 1.38).
+constexpr u32 SMS = 152;  // of a GB300
 template <typename... P, typename... A>
 inline void launch(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchAttribute at{};
@@ -86,9 +87,9 @@ struct NttTables {
 //                 nsrc  > 0 -> sum_j src[j*N + x] * bcst[j] mod q   (basis conversion, Eq. 3)
 //                 (bits 0-15: the source count; bit 16: every source word is
 //                 below 2^40, which with a packed_q target allows 40-bit sums)
-//   pass 2 store: subout == nullptr -> dst[x] = X;
-//                 otherwise subout[x] = (subx[x] - X) * c mod q        (ModDown tail, Eq. 4)
-// Pass 1 writes dst; pass 2 runs in place on dst.
+//   pass 2 store: subx == nullptr -> dst[x] = X;
+//                 otherwise dst[x] = (subx[x] - X) * c mod q          (ModDown tail, Eq. 4)
+// Pass 1 writes dst; pass 2 runs in place on dst.  subx is a plain limb.
 // FwdJob::nsrc bit 17: a copy job, dst[x] = src[x -> x^gal] with gal in c
 // (0: plain copy) and no transform, for the limbs a Decompose passes through
 // unchanged; it rides in the same launch as the transforms.
@@ -104,7 +105,6 @@ struct FwdJob {
     u64* dst;
     const u64* bcst;
     const u64* subx;
-    u64* subout;
     u64 c, c_sh;
     u32 mod;
     u32 nsrc;
@@ -122,22 +122,49 @@ struct InvJob {
     u32 gal;
 };
 
+// An inverse transform with a basis conversion taken off on the way out:
+// dst[x] = X[x] * c - (sum_i csrc[i*N + x] * bcst[i]) * c2 mod q, i < nsrc,
+// X the unscaled inverse.  A ModDown that feeds a Decompose (Alg. 2 lines 6-7
+// and 15-16) needs the coefficients of (x - conv) P^-1, and
+// INTT(x - NTT(conv)) = INTT(x) - conv.
+struct InvConvJob : InvJob {
+    const u64* csrc;
+    const u64* bcst;
+    u64 c2, c2_sh;
+    u32 nsrc;
+    u32 pad;
+};
+// The inverse transforms of `sub` after those of `first`, whose outputs are the
+// sub jobs' csrc; their row passes are one launch.
+void launch_inv_conv(const NttTables& T, const InvJob* first, int nfirst, const InvConvJob* sub, int nsub, cudaStream_t st);
+
 void launch_fwd_ntt(const NttTables& T, const FwdJob* jobs, int njobs, cudaStream_t st);
 void launch_inv_ntt(const NttTables& T, const InvJob* jobs, int njobs, cudaStream_t st);
 
 // out[l][s] = in[l][src_g(s)] for n_limbs limbs (NTT-domain automorphism, Eq. 7).
 void launch_automorphism(const u64* in, u64* out, u32 n_limbs, u32 gal, u32 log_n, cudaStream_t st);
 
-// out[s] = (acc ? out[s] : 0) + a[src_g(s)] + b[s] mod q_l, per limb (b may be null).
+// out[s] = a[src_gal(s)] + b[s] mod q, per limb.
 struct AddJob {
     const u64* a;
     const u64* b;
     u64* out;
     u32 mod;
-    u32 pad;
+    u32 gal;
 };
-void launch_add_gather(const ModC* mods, const AddJob* jobs, int njobs, u32 gal, int accumulate, u32 log_n,
-                       cudaStream_t st);
+void launch_add_gather(const ModC* mods, const AddJob* jobs, int njobs, u32 log_n, cudaStream_t st);
+
+// The giant steps' sum of BSGS: acc0[t][s] += sum_k a_k[t][src_{g_k}(s)] + b0_k[t][s] and
+// acc1[t][s] += sum_k b1_k[t][s] mod q_t, over `level` Q limbs, k < count.
+constexpr int SUM_MAX = 64;
+struct SumArgs {
+    const u64 *a[SUM_MAX], *b0[SUM_MAX], *b1[SUM_MAX];
+    u32 gal[SUM_MAX];
+    u64 *acc0, *acc1;
+    const ModC* mods;
+    u32 count, level, log_n;
+};
+void launch_sum_gather(const SumArgs& a, cudaStream_t st);
 
 // Where word x of digit b of limb t lies: t limb + (x / BLK) blk + b dig + x % BLK.
 // Plain digits [beta][ext][N], or grouped [ext][N/BLK][slots][BLK]: the slots

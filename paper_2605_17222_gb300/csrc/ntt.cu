@@ -138,14 +138,15 @@ ProfScope::~ProfScope() {
 
 namespace {
 
-// Jobs per launch, passed by value: 510 forward jobs (64 bytes each) and the tables fill the
-// 32,764 bytes of kernel parameters; a level-24 Decompose of three polynomials (504 jobs) is one
-// launch.  Launches of up to 60 jobs take a pack of 4 KB: the host copies every byte of the
-// parameters at each launch (1.7 us a launch against 2.7).
-constexpr int MAXJ = 510, SMALLJ = 60;
-static_assert(sizeof(FwdJob) * MAXJ + sizeof(NttTables) <= 32764, "forward jobs exceed the kernel parameter space");
-static_assert(sizeof(InvJob) * MAXJ + sizeof(NttTables) <= 32764, "inverse jobs exceed the kernel parameter space");
-static_assert(sizeof(AddJob) * MAXJ + 64 <= 32764, "add jobs exceed the kernel parameter space");
+// Jobs per launch, passed by value: up to 510, or what fills the 32,764 bytes of kernel parameters
+// beside the tables; a level-24 Decompose of three polynomials (504 jobs) is one launch.  Launches of
+// up to SMALLJ jobs take a small pack: the host copies every byte of the parameters at each launch
+// (1.7 us a launch with 4 KB, 2.7 with 32 KB).
+constexpr int SMALLJ = 60;
+template <typename J>
+constexpr int max_jobs() {
+    return std::min<int>(510, (32764 - 64 - (int)sizeof(NttTables)) / (int)sizeof(J));
+}
 constexpr int THREADS = 256;
 
 template <typename J, int CAP>
@@ -350,17 +351,17 @@ __device__ __forceinline__ void fwd_cols_stages(u64 (&x)[16], u64* sm, u32 u, u3
 // bconv_words save four multiplier slots and pay as many in their second
 // reduction (level-24 LT at N = 2^16, its four column passes: 397 us, 417 with them).
 template <int LOGS, int NS>
-__device__ __forceinline__ void bconv_words96(u64* sm, const FwdJob& J, u32 u, u32 c, u32 col, u32 N, u32 C,
+__device__ __forceinline__ void bconv_words96(u64* sm, const u64* in, const u64* bcst, u32 u, u32 c, u32 col, u32 N, u32 C,
                                               const ModC& m) {
     constexpr u32 S = 1u << LOGS, TPL = S / 16, W = THREADS / TPL;
     u64 cst[NS];
 #pragma unroll
-    for (int j = 0; j < NS; j++) cst[j] = J.bcst[j];
+    for (int j = 0; j < NS; j++) cst[j] = bcst[j];
     const u64 q = m.q;
     const u64 c64 = 0 - q * m.mu_hi;                    // 2^64 mod q (mu_hi = floor(2^64 / q))
     const u64 c63 = (c64 + ((c64 & 1) ? q : 0)) >> 1;   // 2^63 mod q
     const u32 mu32 = (u32)m.mu_hi;
-    const u64* src = J.src + (size_t)u * C + col;
+    const u64* src = in + (size_t)u * C + col;
 #pragma unroll 4
     for (int v = 0; v < 16; v++) {
         const u64* p = src + (size_t)(TPL * v) * C;
@@ -382,13 +383,14 @@ __device__ __forceinline__ void bconv_words96(u64* sm, const FwdJob& J, u32 u, u
 // (N = 2^14 BSGS, 44 column passes: 1014 -> 734 us).  SMALL: sources below 2^40 and a packed_q target,
 // 40-bit sums reduced to [0, 3q); otherwise 60-bit sums, reduced below 5q and
 // brought into [0, 3q).  Either feeds the butterflies.
-template <int LOGS, int NS, bool SMALL>
-__device__ __forceinline__ void bconv_words(u64* sm, const FwdJob& J, u32 ns, u32 u, u32 c, u32 col, u32 N, u32 C,
-                                            const ModC& m) {
-    constexpr u32 S = 1u << LOGS, TPL = S / 16, W = THREADS / TPL, G = NS ? NS : 8;
+// emit(v, r) takes word v's sum r.
+template <int LOGS, int NS, bool SMALL, typename F>
+__device__ __forceinline__ void bconv_words(const u64* in, const u64* bcst, u32 ns, u32 u, u32 col, u32 N, u32 C,
+                                            const ModC& m, F&& emit) {
+    constexpr u32 S = 1u << LOGS, TPL = S / 16, G = NS ? NS : 8;
     typedef typename std::conditional<SMALL, Sum40, Sum60>::type Sum;
     const u64 q = m.q;
-    const u64* src = J.src + (size_t)u * C + col;
+    const u64* src = in + (size_t)u * C + col;
     u32 k0[NS ? NS : 1], k1[NS ? NS : 1];
     auto split_k = [](u64 x, u32& lo, u32& hi) {
         if constexpr (SMALL) lo = (u32)x, hi = (u32)(x >> 32);
@@ -403,7 +405,7 @@ __device__ __forceinline__ void bconv_words(u64* sm, const FwdJob& J, u32 ns, u3
         else return s.value(add, m);
     };
 #pragma unroll
-    for (int j = 0; j < NS; j++) split_k(J.bcst[j], k0[j], k1[j]);
+    for (int j = 0; j < NS; j++) split_k(bcst[j], k0[j], k1[j]);
     // words per step: four where the sources are counted at run time, else one, unrolled four deep
     constexpr int VG = NS ? 1 : 4, VU = NS ? 4 : 1;
 #pragma unroll VU
@@ -430,7 +432,7 @@ __device__ __forceinline__ void bconv_words(u64* sm, const FwdJob& J, u32 ns, u3
 #pragma unroll 2
                 for (u32 j = j0; j < je; j++) {
                     u32 c0, c1;
-                    split_k(J.bcst[j], c0, c1);
+                    split_k(bcst[j], c0, c1);
 #pragma unroll
                     for (int v = 0; v < VG; v++) {
                         u32 d0, d1;
@@ -445,7 +447,7 @@ __device__ __forceinline__ void bconv_words(u64* sm, const FwdJob& J, u32 ns, u3
 #pragma unroll
         for (int v = 0; v < VG; v++) {
             if constexpr (!SMALL) r[v] = r[v] >= 2 * q ? r[v] - 2 * q : r[v];
-            sm[(u + TPL * (v0 + v)) * W + c] = r[v];
+            emit(v0 + v, r[v]);
         }
     }
 }
@@ -491,13 +493,14 @@ __global__ void __launch_bounds__(THREADS, 4) k_fwd_cols(const __grid_constant__
         // basis conversion (Eq. 3) of the thread's 16 words, staged through its
         // own slots of the exchange buffer so that this part stays a compact loop
         const u32 ns = J.nsrc & 0xFFFFu;
+        auto park = [&](int v, u64 r) { sm[(u + TPL * v) * W + c] = r; };
         if (((J.nsrc >> 16) & 1u) && packed_q(q)) {
-            if (ns == 4) bconv_words96<LOGS, 4>(sm, J, u, c, col, N, C, m);
-            else bconv_words<LOGS, 0, true>(sm, J, ns, u, c, col, N, C, m);
+            if (ns == 4) bconv_words96<LOGS, 4>(sm, J.src, J.bcst, u, c, col, N, C, m);
+            else bconv_words<LOGS, 0, true>(J.src, J.bcst, ns, u, col, N, C, m, park);
         } else if (ns == 4) {
-            bconv_words<LOGS, 4, false>(sm, J, ns, u, c, col, N, C, m);
+            bconv_words<LOGS, 4, false>(J.src, J.bcst, ns, u, col, N, C, m, park);
         } else {
-            bconv_words<LOGS, 0, false>(sm, J, ns, u, c, col, N, C, m);
+            bconv_words<LOGS, 0, false>(J.src, J.bcst, ns, u, col, N, C, m, park);
         }
 #pragma unroll
         for (int v = 0; v < 16; v++) x[v] = sm[(u + TPL * v) * W + c];
@@ -580,7 +583,7 @@ __device__ __forceinline__ void fwd_rows_limb(const FwdJob& J, const ModC& m, co
     constexpr u32 S = 1u << LOGS, TPL = S / 16, log_r = LOGN - LOGS;
     const u64 q = m.q;
     const size_t base = (size_t)row * S;
-    const u32 step = SUBMUL ? BLK : fwd_step(J);  // a ModDown's limbs are plain
+    const u32 step = fwd_step(J);
     u64* p = J.dst + blk_off<S>(row, u, step);
     u64 x[16];
 #pragma unroll
@@ -603,8 +606,7 @@ __device__ __forceinline__ void fwd_rows_limb(const FwdJob& J, const ModC& m, co
     __syncwarp();
 #pragma unroll
     for (int v = 0; v < 16; v++) {
-        const u32 xi = u + TPL * v;
-        const u64 y = sr[pad16(xi)];
+        const u64 y = sr[pad16(u + TPL * v)];
         u64 val;
         if constexpr (AR == 2) {  // below 68q < 2^48 -> [0, 3q)
             val = red3_small(y, q, (u32)m.mu_hi);
@@ -617,7 +619,7 @@ __device__ __forceinline__ void fwd_rows_limb(const FwdJob& J, const ModC& m, co
             val = canon4(y, q);
         }
         if constexpr (SUBMUL) {
-            J.subout[base + xi] = mul_shoup(sub_mod(sx[v], val, q), J.c, J.c_sh, q);
+            p[row_off<TPL>(v, step)] = mul_shoup(sub_mod(sx[v], val, q), J.c, J.c_sh, q);
         } else {
             p[row_off<TPL>(v, step)] = val;
         }
@@ -632,9 +634,10 @@ constexpr size_t fwd_rows_smem() {
 }
 
 // Three CTAs per SM (80 registers; measured faster than four at 64).
-template <int LOGN, int LOGS, bool SUBMUL, int CAP>
+// TAIL: 0 no job has a ModDown tail, 1 every one, 2 some.
+template <int LOGN, int LOGS, int TAIL, int CAP>
 __global__ void __launch_bounds__(THREADS, 3) k_fwd_rows(const __grid_constant__ NttTables T,
-                                                      const __grid_constant__ Jobs<FwdJob, CAP> jobs) {
+                                                      const __grid_constant__ Jobs<FwdJob, CAP> jobs, u32 j0) {
     constexpr u32 S = 1u << LOGS, TPL = S / 16, B = THREADS / TPL, SP = S + S / 16;
     constexpr u32 N = 1u << LOGN, log_r = LOGN - LOGS;
     extern __shared__ __align__(16) u64 dsm[];
@@ -642,7 +645,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_fwd_rows(const __grid_constant__
     ulonglong2* t1s = (ulonglong2*)(dsm + B * SP);
     const u32 u = threadIdx.x % TPL, rl = threadIdx.x / TPL;
     const u32 row = blockIdx.x * B + rl;
-    const FwdJob& J = jobs.j[blockIdx.y];
+    const FwdJob& J = jobs.j[j0 + blockIdx.y];
     if (J.nsrc & FWD_COPY) {  // copied by the column pass
         pdl_wait();
         return;
@@ -654,9 +657,14 @@ __global__ void __launch_bounds__(THREADS, 3) k_fwd_rows(const __grid_constant__
     fwd_rows_stage_twiddles<LOGS>(tw, u, row, log_r, t1);
     cp_async_commit();
     pdl_wait();
-    if (small_q(m.q)) fwd_rows_limb<LOGN, LOGS, SUBMUL, 2>(J, m, tw, sr, t1, u, row);
-    else if (m.q < FWD_GROW_MAX) fwd_rows_limb<LOGN, LOGS, SUBMUL, 1>(J, m, tw, sr, t1, u, row);
-    else fwd_rows_limb<LOGN, LOGS, SUBMUL, 0>(J, m, tw, sr, t1, u, row);
+    auto limb = [&](auto submul) {
+        constexpr bool SUBMUL = decltype(submul)::value;
+        if (small_q(m.q)) fwd_rows_limb<LOGN, LOGS, SUBMUL, 2>(J, m, tw, sr, t1, u, row);
+        else if (m.q < FWD_GROW_MAX) fwd_rows_limb<LOGN, LOGS, SUBMUL, 1>(J, m, tw, sr, t1, u, row);
+        else fwd_rows_limb<LOGN, LOGS, SUBMUL, 0>(J, m, tw, sr, t1, u, row);
+    };
+    if (TAIL == 1 || (TAIL == 2 && J.subx)) limb(std::true_type{});
+    else limb(std::false_type{});
 }
 
 // Sets a kernel's dynamic shared memory limit once per device.
@@ -760,16 +768,17 @@ __device__ __forceinline__ void inv_cols_stages(u64 (&x)[16], u64* sm, u32 u, u3
     }
 }
 
-template <int LOGN, int LOGS, int CAP>
+template <int LOGN, int LOGS, int CAP, typename J_T>
 __global__ void __launch_bounds__(THREADS, 3) k_inv_cols(const __grid_constant__ NttTables T,
-                                                      const __grid_constant__ Jobs<InvJob, CAP> jobs) {
+                                                      const __grid_constant__ Jobs<J_T, CAP> jobs) {
     constexpr u32 S = 1u << LOGS, TPL = S / 16, W = THREADS / TPL;
     __shared__ u64 sm[S * W];
     __shared__ __align__(16) ulonglong2 ts[S];
     constexpr u32 N = 1u << LOGN, C = N >> LOGS;
+    constexpr bool CONV = std::is_same<J_T, InvConvJob>::value;
     const u32 c = threadIdx.x % W, u = threadIdx.x / W;
     const u32 col = blockIdx.x * W + c;
-    const InvJob& J = jobs.j[blockIdx.y];
+    const J_T& J = jobs.j[blockIdx.y];
     const u64 q = T.mods[J.mod].q;
     const ulonglong2* tw = T.ipsi + (size_t)J.mod * N;
     // the S - 1 twiddle pairs of the column stages (indices 1 .. S - 1), copied while the words load
@@ -782,9 +791,22 @@ __global__ void __launch_bounds__(THREADS, 3) k_inv_cols(const __grid_constant__
     cp_async_wait_all();
     __syncthreads();
     inv_cols_stages<LOGS>(x, sm, u, c, ts, q);
-    // the scaling: mul_shoup reduces any 64-bit word fully
+    if constexpr (CONV) {
+        const ModC m = T.mods[J.mod];
+        __syncthreads();  // the exchange has been read: its slots park the words, four of which meet their sums at a time
 #pragma unroll
-    for (int v = 0; v < 16; v++) J.dst[(size_t)(u + TPL * v) * C + col] = mul_shoup(x[v], J.c, J.c_sh, q);
+        for (int v = 0; v < 16; v++) sm[(u + TPL * v) * W + c] = x[v];
+        auto emit = [&](int v, u64 r) {
+            const u64 y = mul_shoup_lazy(sm[(u + TPL * v) * W + c], J.c, J.c_sh, q) + 2 * q -
+                          mul_shoup_lazy(r, J.c2, J.c2_sh, q);  // below 4q
+            J.dst[(size_t)(u + TPL * v) * C + col] = canon4(y, q);
+        };
+        bconv_words<LOGS, 0, false>(J.csrc, J.bcst, J.nsrc, u, col, N, C, m, emit);
+    } else {
+        // the scaling: mul_shoup reduces any 64-bit word fully
+#pragma unroll
+        for (int v = 0; v < 16; v++) J.dst[(size_t)(u + TPL * v) * C + col] = mul_shoup(x[v], J.c, J.c_sh, q);
+    }
 }
 
 __global__ void k_automorphism(const u64* __restrict__ in, u64* __restrict__ out, u32 gal, u32 log_n) {
@@ -796,18 +818,29 @@ __global__ void k_automorphism(const u64* __restrict__ in, u64* __restrict__ out
 }
 
 template <int CAP>
-__global__ void k_add_gather(const ModC* __restrict__ mods, const __grid_constant__ Jobs<AddJob, CAP> jobs, u32 gal,
-                             int acc, u32 log_n) {
+__global__ void k_add_gather(const ModC* __restrict__ mods, const __grid_constant__ Jobs<AddJob, CAP> jobs,
+                             u32 log_n) {
     const u32 N = 1u << log_n;
     const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
     const AddJob& J = jobs.j[blockIdx.y];
     const u64 q = mods[J.mod].q;
     pdl_wait();
-    u64 v = J.a[gal ? auto_src(s, gal, log_n) : s];
-    if (J.b) v = add_mod(v, J.b[s], q);
-    if (acc) v = add_mod(v, J.out[s], q);
-    J.out[s] = v;
+    J.out[s] = add_mod(J.a[J.gal ? auto_src(s, J.gal, log_n) : s], J.b[s], q);
+}
+
+__global__ void k_sum_gather(const __grid_constant__ SumArgs a) {
+    const u32 s = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;
+    const size_t o = ((size_t)t << a.log_n);
+    const u64 q = a.mods[t].q;
+    pdl_wait();
+    u64 v0 = a.acc0[o + s], v1 = a.acc1[o + s];
+    for (u32 k = 0; k < a.count; k++) {
+        v0 = add_mod(v0, add_mod(a.a[k][o + auto_src(s, a.gal[k], a.log_n)], a.b0[k][o + s], q), q);
+        v1 = add_mod(v1, a.b1[k][o + s], q);
+    }
+    a.acc0[o + s] = v0;
+    a.acc1[o + s] = v1;
 }
 
 template <int CAP, typename J, typename F>
@@ -818,6 +851,7 @@ void with_pack(const J* jobs, int n, F&& f) {
 }
 template <typename J, typename F>
 void for_chunks(const J* jobs, int njobs, F&& f) {
+    constexpr int MAXJ = max_jobs<J>();
     for (int s = 0; s < njobs; s += MAXJ) {
         const int n = std::min(MAXJ, njobs - s);
         if (n <= SMALLJ) with_pack<SMALLJ>(jobs + s, n, f);
@@ -826,7 +860,7 @@ void for_chunks(const J* jobs, int njobs, F&& f) {
 }
 
 template <int LR, int LC, int CAP>
-void fwd_impl(const NttTables& T, const Jobs<FwdJob, CAP>& p, int n, bool bconv, bool submul, cudaStream_t st) {
+void fwd_impl(const NttTables& T, const Jobs<FwdJob, CAP>& p, int n, bool bconv, cudaStream_t st) {
     const u32 N = 1u << T.log_n;
     const dim3 g1((N >> LR) / (THREADS / ((1u << LR) / 16)), n), g2((N >> LC) / (THREADS / ((1u << LC) / 16)), n);
     int nt = 0;  // transformed limbs (copy jobs aside)
@@ -845,42 +879,51 @@ void fwd_impl(const NttTables& T, const Jobs<FwdJob, CAP>& p, int n, bool bconv,
         if (!nt) return;  // copies only
         ProfScope ps(K_FWD_ROWS, st, 0, half * LC);
         constexpr size_t sm = fwd_rows_smem<LC>();
-        static std::atomic<uint64_t> lim_t{0}, lim_f{0};
-        if (submul) {
-            smem_limit(k_fwd_rows<LR + LC, LC, true, CAP>, sm, lim_t);
-            launch(true, k_fwd_rows<LR + LC, LC, true, CAP>, g2, THREADS, sm, st, T, p);
+        auto rows = [&](auto tail, int j0, int count) {
+            constexpr int TAIL = decltype(tail)::value;
+            static std::atomic<uint64_t> lim{0};
+            if (count <= 0) return;
+            smem_limit(k_fwd_rows<LR + LC, LC, TAIL, CAP>, sm, lim);
+            launch(true, k_fwd_rows<LR + LC, LC, TAIL, CAP>, dim3(g2.x, count), THREADS, sm, st, T, p, (u32)j0);
+        };
+        // The jobs with a ModDown tail are the last ones.  One kernel with both bodies is 6% slower
+        // (N = 2^16 level 24: 324 us for 304) and saves a launch of 7 us: for grids that leave SMs idle.
+        int plain = n;
+        while (plain > 0 && p.j[plain - 1].subx) plain--;
+        if (CAP == SMALLJ && plain > 0 && plain < n && g2.x * n <= SMS) {
+            rows(std::integral_constant<int, 2>{}, 0, n);
         } else {
-            smem_limit(k_fwd_rows<LR + LC, LC, false, CAP>, sm, lim_f);
-            launch(true, k_fwd_rows<LR + LC, LC, false, CAP>, g2, THREADS, sm, st, T, p);
+            rows(std::integral_constant<int, 0>{}, 0, plain);
+            rows(std::integral_constant<int, 1>{}, plain, n - plain);
         }
     }
 }
 
 template <int LR, int LC, int CAP>
-void inv_impl(const NttTables& T, const Jobs<InvJob, CAP>& p, int n, bool gather, cudaStream_t st) {
+void inv_rows_impl(const NttTables& T, const Jobs<InvJob, CAP>& p, int n, bool gather, cudaStream_t st) {
     const u32 N = 1u << T.log_n;
-    const dim3 g1((N >> LR) / (THREADS / ((1u << LR) / 16)), n), g2((N >> LC) / (THREADS / ((1u << LC) / 16)), n);
-    const double half = (double)n * (N / 2);
-    const bool early = g2.x * g2.y < 64;
-    {
-        ProfScope ps(K_INV_ROWS, st, 0, half * LC);
-        if (gather) launch(early, k_inv_rows<LR + LC, LC, true, CAP>, g2, THREADS, 0, st, T, p);
-        else launch(early, k_inv_rows<LR + LC, LC, false, CAP>, g2, THREADS, 0, st, T, p);
-    }
-    {
-        ProfScope ps(K_INV_COLS, st, 0, half * LR);
-        launch(true, k_inv_cols<LR + LC, LR, CAP>, g1, THREADS, 0, st, T, p);
-    }
+    const dim3 g((N >> LC) / (THREADS / ((1u << LC) / 16)), n);
+    const bool early = g.x * g.y < 64;
+    ProfScope ps(K_INV_ROWS, st, 0, (double)n * (N / 2) * LC);
+    if (gather) launch(early, k_inv_rows<LR + LC, LC, true, CAP>, g, THREADS, 0, st, T, p);
+    else launch(early, k_inv_rows<LR + LC, LC, false, CAP>, g, THREADS, 0, st, T, p);
+}
+template <int LR, int LC, int CAP, typename J>
+void inv_cols_impl(const NttTables& T, const Jobs<J, CAP>& p, int n, cudaStream_t st) {
+    const u32 N = 1u << T.log_n;
+    const dim3 g((N >> LR) / (THREADS / ((1u << LR) / 16)), n);
+    ProfScope ps(K_INV_COLS, st, 0, (double)n * (N / 2) * LR);
+    launch(true, k_inv_cols<LR + LC, LR, CAP, J>, g, THREADS, 0, st, T, p);
 }
 
 // N = 2^log_n is viewed as R x C with log R = ceil(log_n / 2).
-#define NTT_DISPATCH(IMPL, ...)                                   \
-    switch (T.log_n) {                                            \
-        case 12: IMPL<6, 6>(T, p, n, __VA_ARGS__, st); break;    \
-        case 13: IMPL<7, 6>(T, p, n, __VA_ARGS__, st); break;    \
-        case 14: IMPL<7, 7>(T, p, n, __VA_ARGS__, st); break;    \
-        case 15: IMPL<8, 7>(T, p, n, __VA_ARGS__, st); break;    \
-        default: IMPL<8, 8>(T, p, n, __VA_ARGS__, st); break; /* 16: contexts take 12..16 */ \
+#define NTT_DISPATCH(IMPL, ...)                                  \
+    switch (T.log_n) {                                           \
+        case 12: IMPL<6, 6>(T, p, n, __VA_ARGS__); break;        \
+        case 13: IMPL<7, 6>(T, p, n, __VA_ARGS__); break;        \
+        case 14: IMPL<7, 7>(T, p, n, __VA_ARGS__); break;        \
+        case 15: IMPL<8, 7>(T, p, n, __VA_ARGS__); break;        \
+        default: IMPL<8, 8>(T, p, n, __VA_ARGS__); break; /* 16: contexts take 12..16 */ \
     }
 
 // ------------------------------------------------------------------ integer-rate probes
@@ -939,28 +982,49 @@ __global__ void __launch_bounds__(PROBE_THREADS, 4) k_probe_bfly(const ulonglong
 
 void launch_fwd_ntt(const NttTables& T, const FwdJob* jobs, int njobs, cudaStream_t st) {
     if (njobs <= 0) return;
-    // every transform job of a launch is of one kind (copy jobs may join any)
-    bool bconv = false, submul = false, transforms = false;
+    // the transform jobs of a launch all convert a basis on load or none does (copy jobs may join any);
+    // those with a ModDown tail come last
+    bool bconv = false, transforms = false;
     for (int i = 0; i < njobs; i++)
         if (!(jobs[i].nsrc & FWD_COPY)) {
             bconv = (jobs[i].nsrc & 0xFFFFu) > 0;
             transforms = true;
-            submul = jobs[i].subout != nullptr;
             break;
         }
     for_chunks(jobs, njobs, [&](const auto& p, int n) {
-        NTT_DISPATCH(fwd_impl, bconv, submul);
+        NTT_DISPATCH(fwd_impl, bconv, st);
         count_launch(transforms ? 2 : 1);
+    });
+}
+
+static void launch_inv_rows(const NttTables& T, const InvJob* jobs, int njobs, cudaStream_t st) {
+    const bool gather = jobs[0].gal != 0;
+    for_chunks(jobs, njobs, [&](const auto& p, int n) {
+        NTT_DISPATCH(inv_rows_impl, gather, st);
+        count_launch();
+    });
+}
+template <typename J>
+static void launch_inv_cols(const NttTables& T, const J* jobs, int njobs, cudaStream_t st) {
+    for_chunks(jobs, njobs, [&](const auto& p, int n) {
+        NTT_DISPATCH(inv_cols_impl, st);
+        count_launch();
     });
 }
 
 void launch_inv_ntt(const NttTables& T, const InvJob* jobs, int njobs, cudaStream_t st) {
     if (njobs <= 0) return;
-    const bool gather = jobs[0].gal != 0;
-    for_chunks(jobs, njobs, [&](const auto& p, int n) {
-        NTT_DISPATCH(inv_impl, gather);
-        count_launch(2);
-    });
+    launch_inv_rows(T, jobs, njobs, st);
+    launch_inv_cols(T, jobs, njobs, st);
+}
+
+void launch_inv_conv(const NttTables& T, const InvJob* first, int nfirst, const InvConvJob* sub, int nsub,
+                     cudaStream_t st) {
+    std::vector<InvJob> rows(first, first + nfirst);
+    rows.insert(rows.end(), sub, sub + nsub);  // their InvJob part
+    launch_inv_rows(T, rows.data(), (int)rows.size(), st);
+    launch_inv_cols(T, first, nfirst, st);
+    launch_inv_cols(T, sub, nsub, st);
 }
 
 void launch_automorphism(const u64* in, u64* out, u32 n_limbs, u32 gal, u32 log_n, cudaStream_t st) {
@@ -1025,15 +1089,20 @@ cudaError_t probe_int_rates(u32 blocks, double* macs_per_s, double* butterflies_
     return cudaSuccess;
 }
 
-void launch_add_gather(const ModC* mods, const AddJob* jobs, int njobs, u32 gal, int accumulate, u32 log_n,
-                       cudaStream_t st) {
+void launch_add_gather(const ModC* mods, const AddJob* jobs, int njobs, u32 log_n, cudaStream_t st) {
     const u32 N = 1u << log_n;
     for_chunks(jobs, njobs, [&](const auto& p, int n) {
         ProfScope ps(K_ADD, st);
-        launch(true, k_add_gather<std::extent<decltype(p.j)>::value>, dim3((N + 255) / 256, n), 256, 0, st, mods, p, gal,
-                   accumulate, log_n);
+        launch(true, k_add_gather<std::extent<decltype(p.j)>::value>, dim3((N + 255) / 256, n), 256, 0, st, mods, p,
+               log_n);
         count_launch();
     });
+}
+
+void launch_sum_gather(const SumArgs& a, cudaStream_t st) {
+    ProfScope ps(K_ADD, st);
+    launch(true, k_sum_gather, dim3((1u << a.log_n) / 256, a.level), 256, 0, st, a);
+    count_launch();
 }
 
 }  // namespace ckks

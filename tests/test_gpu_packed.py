@@ -112,3 +112,30 @@ def test_operands_at_any_word(words):
     for x, y in zip(got, want):
         assert_same(x.numpy(), y.numpy(), f"offset {words}")
     g.close()
+
+
+@pytest.mark.parametrize("params,level,split,algo", [
+    ("n14", 8, (3, 2, 3), "th"),    # ModDown into Decompose as one step
+    ("n14", 5, (9, 2), "bsgs"),     # a partial last digit, rotations in one chunk
+    ("setA", 5, (2, 2, 4), "th"),   # five special limbs
+])
+def test_merged_key_switches_equal_their_steps(params, level, split, algo):
+    """LTs whose key switches run merged or batched, bit for bit with the oracle's step by step."""
+    import oracle.ckks as ock
+    from oracle import lt as olt
+    from paper_2605_17222_gb300 import binding, synth
+
+    ps = synth.param_set(params)
+    octx, g = ock.Ctx(ps), binding.Context.from_params(ps)
+    D = int(np.prod(split))
+    keys = {}
+    for r in olt.rotation_set(algo, D, split, 1, ps.n // 2, 2):
+        keys[r] = np.stack([synth.uniform_mod(11 + r + 1000 * b, "key", ps.moduli, ps.n)
+                            for b in range(2 * octx.beta_max)]).reshape(octx.beta_max, 2, len(ps.moduli), ps.n)
+        g.upload_rotation_key(r, keys[r])
+    f = np.stack([synth.uniform_mod(5 + d, "f", ps.moduli, ps.n) for d in range(D)])
+    ct = np.stack([synth.uniform_mod(7 + c, "ct", ps.q[:level], ps.n) for c in range(2)])
+    want = np.stack(olt.run(octx, algo, (ct[0], ct[1]), f, keys, split, 1, 2)[0])
+    got, _ = g.lt_eval(g.ct_from_host(ct), g.upload_diagonals(f, offset0=2), algo, split)
+    assert_same(got.numpy(), want, f"{params} {algo} {split}")
+    g.close()
