@@ -191,15 +191,11 @@ __device__ __forceinline__ u64 canon4(u64 x, u64 q) {
 // Any 64-bit word -> [0, 2q): the Shoup product by 1 (floor(2^64 / q) = mu_hi).
 __device__ __forceinline__ u64 red2(u64 x, u64 q, u64 mu_hi) { return x - __umul64hi(x, mu_hi) * q; }
 
-// x < 2^50 -> [0, 3q) for 2^32 < q < 2^41, with mu32 = floor(2^64 / q) (below
-// 2^32).  The estimate qe = floor(floor(x / 2^32) mu32 / 2^32) never exceeds
-// floor(x / q) and falls short of it by at most 2: the dropped low word of x
-// is worth below 2^32 / q < 1, mu32's truncation below floor(x / 2^32) / 2^32
-// < 2^-14, and the floor below 1.  One 32 x 32 product and one small product
-// by q, instead of the 64 x 64 high product of red2.
+// Any 64-bit word -> [0, 3q) for 2^32 < q < 2^41, mu32 = floor(2^64 / q) (below
+// 2^32): one 32 x 32 high product and two multiply-adds, instead of the 64 x 64
+// high product of red2.
 __device__ __forceinline__ u64 red3_small(u64 x, u64 q, u32 mu32) {
-    const u64 qe = ((u64)(u32)(x >> 32) * mu32) >> 32;
-    return x - qe * q;
+    return reduce64_40(x, q, mu32);
 }
 __device__ __forceinline__ bool small_q(u64 q) { return q > (1ull << 32) && q < (1ull << 41); }
 
@@ -219,11 +215,24 @@ constexpr u64 FWD_GROW_MAX = 1ull << 57;
 // the four 32 x 32 partial products of b ws the quotient estimate keeps the
 // high one and the high halves of the two middle ones; what it drops carries
 // at most 2 into bit 64, so the estimate is below floor(b ws / 2^64) by at
-// most 2 and the remainder lies in [0, 2q) + [0, 2q).
+// most 2 and the remainder lies in [0, 2q) + [0, 2q).  Spelled out as one chain
+// of 32-bit multiply-adds (b w + qe (2^64 - q) mod 2^64): from the 64-bit
+// expressions the compiler spends a third of the passes' multiplier
+// instructions on moves and carries (level-24 LT at N = 2^16: column passes
+// 407 -> 390 us, row passes 308 -> 305).
 __device__ __forceinline__ u64 mul_shoup_approx(u64 b, u64 w, u64 ws, u64 q) {
-    const u32 b0 = (u32)b, b1 = (u32)(b >> 32), s0 = (u32)ws, s1 = (u32)(ws >> 32);
-    const u64 qe = (u64)b1 * s1 + __umulhi(b0, s1) + __umulhi(b1, s0);
-    return b * w - qe * q;
+    u64 r;
+    asm("{\n\t.reg .u32 b0, b1, s0, s1, w0, w1, n0, n1, e0, e1, t0, t1;\n\t.reg .u64 e, t;\n\t"
+        "mov.b64 {b0, b1}, %1;\n\tmov.b64 {w0, w1}, %2;\n\tmov.b64 {s0, s1}, %3;\n\tmov.b64 {n0, n1}, %4;\n\t"
+        "mul.wide.u32 e, b1, s1;\n\tmov.b64 {e0, e1}, e;\n\t"
+        "mad.hi.cc.u32 e0, b0, s1, e0;\n\taddc.u32 e1, e1, 0;\n\t"
+        "mad.hi.cc.u32 e0, b1, s0, e0;\n\taddc.u32 e1, e1, 0;\n\t"
+        "mul.wide.u32 t, b0, w0;\n\t"
+        "mad.wide.u32 t, e0, n0, t;\n\tmov.b64 {t0, t1}, t;\n\t"
+        "mad.lo.u32 t1, b0, w1, t1;\n\tmad.lo.u32 t1, b1, w0, t1;\n\t"
+        "mad.lo.u32 t1, e0, n1, t1;\n\tmad.lo.u32 t1, e1, n0, t1;\n\t"
+        "mov.b64 %0, {t0, t1};\n\t}" : "=l"(r) : "l"(b), "l"(w), "l"(ws), "l"(0 - q));
+    return r;
 }
 
 template <bool GROW>
@@ -257,18 +266,19 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// Gentleman-Sande butterfly (inverse), lazy (Harvey), for every modulus below
-// 2^62: inputs and outputs in [0, 2q); (a, b) -> (a + b, (a - b) w) mod q up
-// to multiples of q (the lazy Shoup product of a word below 4q is in [0, 2q)).
-// One form for all moduli keeps the passes to a single body: a launch of one
-// or two CTAs per SM fetches a body's fully unrolled code from L2 line by
-// line, and the special primes' small launches (ModDown sources) would
-// otherwise run a body that the big launches never warm.
+// Gentleman-Sande butterfly (inverse), lazy, for every modulus below 2^61:
+// inputs and outputs in [0, 4q); (a, b) -> (a + b, (a - b) w) mod q up to
+// multiples of q (mul_shoup_approx of a word below 8q is in [0, 4q); with the
+// exact quotient and words in [0, 2q) the inverse column passes of a level-24
+// LT took 85 us instead of 77).  One form for all moduli keeps the passes to a
+// single body: a launch of one or two CTAs per SM fetches a body's fully
+// unrolled code from L2 line by line, and the special primes' small launches
+// (ModDown sources) would otherwise run a body that the big launches never warm.
 __device__ __forceinline__ void gs_w(u64& a, u64& b, u64 w, u64 ws, u64 q) {
-    const u64 q2 = 2 * q;
+    const u64 q4 = 4 * q;
     const u64 s = a + b;
-    b = mul_shoup_lazy(a - b + q2, w, ws, q);
-    a = s >= q2 ? s - q2 : s;
+    b = mul_shoup_approx(a - b + q4, w, ws, q);
+    a = s >= q4 ? s - q4 : s;
 }
 __device__ __forceinline__ void gs(u64& a, u64& b, const ulonglong2* tab, u32 idx, u64 q) {
     u64 w, ws;
@@ -680,7 +690,7 @@ void smem_limit(K kernel, size_t bytes, std::atomic<uint64_t>& done) {
 
 // ------------------------------------------------------------------ inverse, row pass
 // GS stages with half-width t = 1..S/2 (m = N/2t, twiddle psi^-brv(m + row S/2t + x/2t)).
-// Words enter below q (canonical) and stay in [0, 2q).
+// Words enter below q (canonical) and stay in [0, 4q).
 template <int LOGS>
 __device__ __forceinline__ void inv_rows_stages(u64 (&x)[16], u64* sr, u32 u, u32 row, u32 N,
                                                 const ulonglong2* tw, u64 q) {
@@ -735,14 +745,14 @@ __global__ void __launch_bounds__(THREADS, 3) k_inv_rows(const __grid_constant__
     __syncwarp();
 #pragma unroll
     for (int v = 0; v < 16; v++) x[v] = sr[pad16(16 * u + v)];
-    inv_rows_stages<LOGS>(x, sr, u, row, N, tw, q);  // [0, 2q)
+    inv_rows_stages<LOGS>(x, sr, u, row, N, tw, q);  // [0, 4q)
 #pragma unroll
     for (int v = 0; v < 16; v++) J.tmp[base + u + TPL * v] = x[v];
 }
 
 // ------------------------------------------------------------------ inverse, column pass
 // GS stages with half-width C*t_r, t_r = 1..S/2 (m = S/2t_r, twiddle psi^-brv(m + r/2t_r)),
-// then the scaling by c (N^-1 and any per-limb constant).  Words enter and stay in [0, 2q).
+// then the scaling by c (N^-1 and any per-limb constant).  Words enter and stay in [0, 4q).
 // ts: the pass's twiddle pairs 0 .. S - 1, staged in shared memory.
 template <int LOGS>
 __device__ __forceinline__ void inv_cols_stages(u64 (&x)[16], u64* sm, u32 u, u32 c, const ulonglong2* ts, u64 q) {
