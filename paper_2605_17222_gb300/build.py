@@ -10,7 +10,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libckkslt.so")
 SOURCES = (["host.cu", "ntt.cu", "ks.cu"]
-           + [f"diag_mac_{k3}_{ctas}.cu" for k3, ctas in ((1, 4), (2, 4), (4, 4), (4, 3), (8, 3), (8, 2))])
+           + [f"diag_mac_{k3}_{cls}.cu" for k3 in (1, 2, 4, 8) for cls in ("packed", "wide")])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
               "--expt-relaxed-constexpr", "-I", os.path.join(HERE, "..", "include")] + ARCH

@@ -1,6 +1,6 @@
 // The staged diagonal multiply-accumulate kernel (K6), instantiated per number
-// of outer indices and CTAs per SM in diag_mac_<K3>_<MINB>.cu so that the
-// instances compile in parallel.
+// of outer indices and class of limbs in diag_mac_<K3>_{packed,wide}.cu so that
+// the instances compile in parallel.
 #pragma once
 #include "kernels.h"
 #include "mbar.cuh"
@@ -31,7 +31,7 @@ namespace {
 // WS_MAX_STAGES; the packed limbs' stages are a quarter smaller, so they get
 // more).
 //
-// At the N = 2^16 (1,64,4) split, 10.3 GB of keys and diagonals: 1.86 ms (2.45
+// At the N = 2^16 (1,64,4) split, 10.3 GB of keys and diagonals: 1.78 ms (2.45
 // before: unpacked, 17 copies per step issued from the lanes of a warp,
 // 96-bit carry chains).  The copies alone take 1.13 ms for the 23 packed limbs
 // (6.7 TB/s), the arithmetic alone 1.2; the multiplier pipe is about 70% busy.
@@ -295,9 +295,17 @@ __host__ __device__ inline u32 ws_stage(bool packed, u32 k3, u32 beta, u32 beta_
     return k3 * diag_blk(packed) + (beta + 1) * BLK * 8 + (kb > BLK * 8 ? kb : BLK * 8);
 }
 
+// Packed and wide limbs are two launches: each class has the registers and the
+// CTAs per SM that suit its body (K3 = 4: 96 registers and four CTAs, or 128
+// and three), and neither keeps the other's code (one kernel for both: 1.86 ms
+// at (1,64,4), Set-A 1.09; split: 1.78 and 1.03).  The wide limbs go first and
+// the packed ones are launched early behind them (they read nothing that the
+// first launch writes); `join` makes the last CTA wait, at its end, for the
+// launch before, so that a kernel that waits for this one has both.
 // ring: bytes of dynamic shared memory for the stages; the j table follows.
-template <int K3, int BETA, int MINB>
-__global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_constant__ DiagMacArgs a, u32 ring) {
+template <int K3, int BETA, int MINB, bool PACKED>
+__global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_constant__ DiagMacArgs a, u32 ring,
+                                                                 bool join) {
     constexpr u32 RB = BLK * 8;  // bytes of a run of words
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) u64 full_bar[WS_MAX_STAGES];
@@ -308,12 +316,12 @@ __global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_c
     const u32 bidx = blockIdx.x % a.batch;
     const u32 run = blockIdx.x / a.batch;
     const size_t ou = bidx * a.bs_u;
-    const u32 t = blockIdx.y;
+    const u32 t = a.limbs[PACKED ? blockIdx.y : a.n_packed + blockIdx.y];
     const u32 k_first = blockIdx.z * K3;
     const u32 k_count = min((u32)K3, a.n3 - k_first);
     const u32 gmod = t < a.level ? t : a.L + (t - a.level);
     const ModC m = a.mods[gmod];
-    const bool packed = packed_q(m.q);
+    constexpr bool packed = PACKED;
     const size_t tN = (size_t)t * N;
     const u32 n1 = a.n1, n2 = a.n2, n1n2 = n1 * n2;
     constexpr u32 beta = BETA;  // a.beta, or 0 without a middle layer
@@ -343,7 +351,8 @@ __global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_c
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    pdl_wait();
+    if (!join) pdl_wait();
+    else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __syncthreads();
     volatile u32* abort = &abort_flag;
 
@@ -402,6 +411,7 @@ __global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_c
         }
         __syncwarp();
         nbar_sync(1, WS_THREADS);  // every thread of the CTA reaches this once
+        if (join && blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) pdl_wait();
         if (*abort && l == BLK) {
             // drain: the last phase issued into each stage (the earlier ones completed and were consumed)
             for (u32 it = issued > ns ? issued - ns : 0; it < issued; it++)
@@ -416,28 +426,31 @@ __global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_c
     const u64 lc = lift_limb ? a.lift_c[gmod] : 0, lsh = lift_limb ? a.lift_sh[gmod] : 0;
     const WsCtx c{a, smem, full_bar, empty_bar, abort, jtab, s, l, k_first, k_count, ns, stage, off_a,
                   ou + tN + s, lift_limb, lc, lsh, m};
-    if (packed) ws_compute<K3, BETA, C40>(c);
-    else if (m.bits <= 55) ws_compute<K3, BETA, C55>(c);
-    else ws_compute<K3, BETA, C60>(c);
+    if constexpr (PACKED) {
+        ws_compute<K3, BETA, C40>(c);
+    } else {
+        if (m.bits <= 55) ws_compute<K3, BETA, C55>(c);
+        else ws_compute<K3, BETA, C60>(c);
+    }
 }
 
-// Launches k_diag_mac_ws<K3, BETA, MINB> with the ring that MINB CTAs per SM
-// leave room for; false if a stage pair does not fit, so that the plain kernel
-// runs.  The dynamic shared-memory limit is a per-device function attribute:
-// set once per device (threads may race to set it; the call is idempotent).  A
-// device that refuses it falls back too, and the error the refusal left is
-// cleared so that a later status check does not see it.
+// Launches k_diag_mac_ws on one class of limbs, with the ring that MINB CTAs
+// per SM leave room for; false if two stages do not fit, so that the plain
+// kernel runs.  The dynamic shared-memory limit is a per-device function
+// attribute: set once per device (threads may race to set it; the call is
+// idempotent).  A device that refuses it falls back too, and the error the
+// refusal left is cleared so that a later status check does not see it.
 constexpr u32 SM_SMEM = 227 * 1024;
 
-template <int K3, int BETA, int MINB>
-bool try_ws(const DiagMacArgs& a, cudaStream_t st) {
+template <int K3, int BETA, int MINB, bool PACKED>
+bool try_ws(const DiagMacArgs& a, bool join, cudaStream_t st) {
     constexpr u32 beta = BETA;
     const u32 N = 1u << a.log_n;
     // one CTA's share, less the 1 KB that the system takes per CTA and the static barriers
     const u32 tab = (4 * a.n2 + 15) & ~15u, share = SM_SMEM / MINB - 1024 - 256;
     if (tab >= share) return false;
     const u32 ring = (share - tab) & ~127u;
-    if (ring < 2 * ws_stage(false, K3, beta, a.beta_max) || ring < 2 * ws_stage(true, K3, beta, a.beta_max)) return false;
+    if (ring < 2 * ws_stage(PACKED, K3, beta, a.beta_max)) return false;
     static std::atomic<uint64_t> attr_set{0}, attr_bad{0};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
@@ -447,7 +460,7 @@ bool try_ws(const DiagMacArgs& a, cudaStream_t st) {
     const uint64_t bit = 1ull << dev;
     if (attr_bad.load(std::memory_order_relaxed) & bit) return false;
     if (!(attr_set.load(std::memory_order_acquire) & bit)) {
-        if (cudaFuncSetAttribute(k_diag_mac_ws<K3, BETA, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(k_diag_mac_ws<K3, BETA, MINB, PACKED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(SM_SMEM / MINB - 1024 - 256)) != cudaSuccess) {
             cudaGetLastError();
             attr_bad.fetch_or(bit, std::memory_order_relaxed);
@@ -455,25 +468,32 @@ bool try_ws(const DiagMacArgs& a, cudaStream_t st) {
         }
         attr_set.fetch_or(bit, std::memory_order_release);
     }
-    const dim3 grid((N / BLK) * a.batch, a.ext, (a.n3 + K3 - 1) / K3);
-    launch(false, k_diag_mac_ws<K3, BETA, MINB>, grid, WS_THREADS, ring + tab, st, a, ring);
+    const dim3 grid((N / BLK) * a.batch, PACKED ? a.n_packed : a.ext - a.n_packed, (a.n3 + K3 - 1) / K3);
+    launch(join, k_diag_mac_ws<K3, BETA, MINB, PACKED>, grid, WS_THREADS, ring + tab, st, a, ring, join);
     return true;
 }
 
 }  // namespace
 
-template <int K3, int MINB>
-bool launch_ws(const DiagMacArgs& a, cudaStream_t st) {
+// CTAs per SM.  More CTAs are more warps and more independent rings, as long as
+// the body keeps its registers.  Four outer indices at N = 2^16 (1,64,4), packed:
+// 1.87 ms with four CTAs, 2.17 with five; eight at N = 2^15 (1,12,8): 154 us with
+// three, 169 with two.  The wide limbs' body takes more: 54-bit moduli, eight
+// outer indices, 0.67 ms with two, 0.78 with three; at N = 2^16 (four) 1.87 with
+// three for them and 1.89 with four.
+template <int K3, bool PACKED>
+bool launch_ws(const DiagMacArgs& a, bool join, cudaStream_t st) {
+    constexpr int MINB = K3 >= 8 ? (PACKED ? 3 : 2) : K3 == 4 && !PACKED ? 3 : 4;
     switch (a.n2 == 1 ? 0 : a.beta) {
-        case 0: return try_ws<K3, 0, MINB>(a, st);
-        case 1: return try_ws<K3, 1, MINB>(a, st);
-        case 2: return try_ws<K3, 2, MINB>(a, st);
-        case 3: return try_ws<K3, 3, MINB>(a, st);
-        case 4: return try_ws<K3, 4, MINB>(a, st);
-        case 5: return try_ws<K3, 5, MINB>(a, st);
-        case 7: return try_ws<K3, 7, MINB>(a, st);
-        case 8: return try_ws<K3, 8, MINB>(a, st);
-        case 6: return try_ws<K3, 6, MINB>(a, st);
+        case 0: return try_ws<K3, 0, MINB, PACKED>(a, join, st);
+        case 1: return try_ws<K3, 1, MINB, PACKED>(a, join, st);
+        case 2: return try_ws<K3, 2, MINB, PACKED>(a, join, st);
+        case 3: return try_ws<K3, 3, MINB, PACKED>(a, join, st);
+        case 4: return try_ws<K3, 4, MINB, PACKED>(a, join, st);
+        case 5: return try_ws<K3, 5, MINB, PACKED>(a, join, st);
+        case 6: return try_ws<K3, 6, MINB, PACKED>(a, join, st);
+        case 7: return try_ws<K3, 7, MINB, PACKED>(a, join, st);
+        case 8: return try_ws<K3, 8, MINB, PACKED>(a, join, st);
         default: return false;
     }
 }

@@ -627,9 +627,13 @@ DiagMacArgs dm_base(ckks_ctx* C, u32 level, bool with_p, const ckks_diags* f, u3
     a.beta = C->beta(level);
     a.beta_max = C->beta_max;
     a.log_n = C->log_n;
-    u32 packed = 0;
-    for (u32 t = 0; t < a.ext; t++) packed += packed_q(C->mods[C->gmod(level, t)]) ? 1 : 0;
-    a.wide = 2 * packed < a.ext;
+    if (a.ext > (u32)DM_MAX_LIMBS) fail(CKKS_EINVAL, "more than 256 limbs in the extended basis");
+    for (int wide = 0; wide < 2; wide++)
+        for (u32 t = 0, n = wide ? a.n_packed : 0; t < a.ext; t++)
+            if (packed_q(C->mods[C->gmod(level, t)]) == !wide) {
+                a.limbs[n++] = (unsigned char)t;
+                if (!wide) a.n_packed = n;
+            }
     a.err = (u32*)C->d_err.p;
     a.wait_ns = C->dbg_wait_ns;
     a.starve_step = C->dbg_starve_step;

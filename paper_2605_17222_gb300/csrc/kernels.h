@@ -212,6 +212,7 @@ constexpr int DM_MAX_N1 = 64;
 constexpr int DM_MAX_N2 = 1024;
 constexpr int DM_MAX_K3 = 8;   // giant indices per thread (grid.z covers the rest)
 constexpr int DM_MAX_N3 = 64;
+constexpr int DM_MAX_LIMBS = 256;
 constexpr int DM_MAX_B = 16;   // ciphertexts per batched launch
 struct DiagMacArgs {
     const ModC* mods;
@@ -242,7 +243,9 @@ struct DiagMacArgs {
     // Tile (0 = default): outer indices per CTA, a power of two below the
     // next power of two >= n3, at most 8.  Results do not depend on it.
     u32 tile_k3;
-    u32 wide;  // most limbs are wide (not packed_q)
+    // the limbs t < ext: the packed_q ones, then the wide ones
+    u32 n_packed;
+    unsigned char limbs[DM_MAX_LIMBS];
     // Batch of ciphertexts sharing the diagonals and keys: ciphertext b uses
     // X[i] + b*bs_x, B[i] + b*bs_b, c1[b] and U0/U1[k] + b*bs_u.  CTAs of the
     // same (limb, run) for different b are adjacent in the grid, so the
@@ -252,10 +255,10 @@ struct DiagMacArgs {
     const u64* c1[DM_MAX_B];
 };
 void launch_diag_mac(const DiagMacArgs& a, cudaStream_t st);
-// Its staged kernel with K3 (1, 2, 4 or 8) outer indices per CTA and MINB CTAs
-// per SM, or false if a shape does not fit (diag_mac.cuh).
-template <int K3, int MINB>
-bool launch_ws(const DiagMacArgs& a, cudaStream_t st);
+// Its staged kernel on the packed or the wide limbs, K3 (1, 2, 4 or 8) outer
+// indices per CTA, or false if a shape does not fit (diag_mac.cuh).
+template <int K3, bool PACKED>
+bool launch_ws(const DiagMacArgs& a, bool join, cudaStream_t st);
 void launch_wait_selftest(u32* err, u64 limit_ns, cudaStream_t st);
 
 uint64_t launches();

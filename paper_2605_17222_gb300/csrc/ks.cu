@@ -19,6 +19,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 namespace ckks {
 namespace {
@@ -254,12 +255,12 @@ __global__ void __launch_bounds__(BLK) k_ks_any(const __grid_constant__ KsArgs a
 // This plain form reads its operands straight from global memory; it runs the
 // shapes whose stages do not fit the staged kernel below (more than eight digits).
 template <int K3>
-__global__ void __launch_bounds__(THREADS, 2) k_diag_mac(const __grid_constant__ DiagMacArgs a) {
+__global__ void __launch_bounds__(THREADS, 2) k_diag_mac(const __grid_constant__ DiagMacArgs a, u32 l0) {
     const u32 N = 1u << a.log_n;
     const u32 bidx = blockIdx.x % a.batch;
     const u32 s = (blockIdx.x / a.batch) * THREADS + threadIdx.x;
     const size_t ox = bidx * a.bs_x, ob = bidx * a.bs_b, ou = bidx * a.bs_u;
-    const u32 t = blockIdx.y;
+    const u32 t = a.limbs[l0 + blockIdx.y];
     if (s >= N) return;
     const u32 k_first = blockIdx.z * K3;
     const u32 k_count = min((u32)K3, a.n3 - k_first);
@@ -458,33 +459,29 @@ void launch_diag_mac(const DiagMacArgs& a, cudaStream_t st) {
     const double macs = (double)N * a.batch * a.ext *
                         (2.0 * n1n2 * a.n3 + 2.0 * beta_mid * grid.z * (n1n2 - a.n1));
     ProfScope ps(K_DIAG_MAC, st, macs);
-    // CTAs per SM.  More CTAs are more warps and more independent rings, and
-    // the packed limbs' 96-register body wants them (four outer indices, N =
-    // 2^16 (1,64,4): 1.86 ms against 1.89 with three; eight, N = 2^15 (1,12,8):
-    // 163 us with three, 186 with two); the wide limbs' body spills there
-    // (54-bit moduli, four: 1.10 against 1.15 ms; eight: 0.67 against 0.78 ms).
     // Bulk copies read 16-byte aligned runs; a wrapped ciphertext may lie at any word.
     bool aligned = true;
     for (u32 b = 0; b < a.batch; b++) aligned = aligned && ((uintptr_t)a.c1[b] & 15) == 0;
     for (u32 i = 0; i < a.n1; i++) aligned = aligned && (((uintptr_t)a.X[i] | (uintptr_t)a.B[i]) & 15) == 0;
-    bool done = false;
-    if (aligned) switch (k3) {
-        case 1: done = launch_ws<1, 4>(a, st); break;
-        case 2: done = launch_ws<2, 4>(a, st); break;
-        case 4: done = a.wide ? launch_ws<4, 3>(a, st) : launch_ws<4, 4>(a, st); break;
-        default: done = a.wide ? launch_ws<8, 2>(a, st) : launch_ws<8, 3>(a, st); break;
-    }
-    if (done) {
+    auto run = [&](auto k3c, auto packedc, bool join) {
+        constexpr int K3 = decltype(k3c)::value;
+        constexpr bool PACKED = decltype(packedc)::value;
+        const u32 l0 = PACKED ? 0 : a.n_packed, n = PACKED ? a.n_packed : a.ext - a.n_packed;
+        if (!n) return;
+        if (!aligned || !launch_ws<K3, PACKED>(a, join, st))
+            launch(false, k_diag_mac<K3>, dim3(grid.x, n, grid.z), THREADS, 0, st, a, l0);
         count_launch();
-        return;
-    }
+    };
+    auto both = [&](auto k3c) {
+        run(k3c, std::false_type{}, false);
+        run(k3c, std::true_type{}, a.n_packed < a.ext);
+    };
     switch (k3) {
-        case 1: launch(false, k_diag_mac<1>, grid, THREADS, 0, st, a); break;
-        case 2: launch(false, k_diag_mac<2>, grid, THREADS, 0, st, a); break;
-        case 4: launch(false, k_diag_mac<4>, grid, THREADS, 0, st, a); break;
-        default: launch(false, k_diag_mac<8>, grid, THREADS, 0, st, a); break;
+        case 1: both(std::integral_constant<int, 1>{}); break;
+        case 2: both(std::integral_constant<int, 2>{}); break;
+        case 4: both(std::integral_constant<int, 4>{}); break;
+        default: both(std::integral_constant<int, 8>{}); break;
     }
-    count_launch();
 }
 
 }  // namespace ckks

@@ -150,17 +150,31 @@ __device__ __forceinline__ u64 reduce_top(u32 w0, u32 w1, u32 w2, u32 w3, const 
     const u32 a0 = up ? w1 : w0, a1 = up ? w2 : w1, a2 = up ? w3 : w2;
     const u32 x0 = __funnelshift_r(a0, a1, sh), x1 = __funnelshift_r(a1, a2, sh);  // shift modulo 32
     const u32 s0 = (u32)m.mu_s, s1 = (u32)(m.mu_s >> 32);
-    const u64 qe = (u64)x1 * s1 + __umulhi(x0, s1) + __umulhi(x1, s0);
-    return ((u64)w1 << 32 | w0) - qe * m.q;
+    u64 r;
+    asm("{\n\t.reg .u32 n0, n1, e0, e1, t0, t1;\n\t.reg .u64 e, t;\n\t"
+        "mov.b64 {n0, n1}, %7;\n\t"
+        "mul.wide.u32 e, %2, %4;\n\tmov.b64 {e0, e1}, e;\n\t"
+        "mad.hi.cc.u32 e0, %1, %4, e0;\n\taddc.u32 e1, e1, 0;\n\t"
+        "mad.hi.cc.u32 e0, %2, %3, e0;\n\taddc.u32 e1, e1, 0;\n\t"
+        "mov.b64 t, {%5, %6};\n\tmad.wide.u32 t, e0, n0, t;\n\tmov.b64 {t0, t1}, t;\n\t"
+        "mad.lo.u32 t1, e0, n1, t1;\n\tmad.lo.u32 t1, e1, n0, t1;\n\t"
+        "mov.b64 %0, {t0, t1};\n\t}" : "=l"(r) : "r"(x0), "r"(x1), "r"(s0), "r"(s1), "r"(w0), "r"(w1), "l"(0 - m.q));
+    return r;
 }
 
 // x mod q up to 2q, in [0, 3q), for any 64-bit x and 2^32 < q < 2^40
 // (mu32 = floor(2^64 / q) below 2^32): dropping x's low word costs less than
 // 1, mu32's truncation less than 1, the floor less than 1.
+// x + qe (2^64 - q) in three multiplies, spelled out (like Sum40's fold) because
+// the 64-bit expressions leave moves on the multiplier pipe: the diagonal kernel
+// at (1,64,4) takes 1.87 ms with them and 1.78 without.
 __device__ __forceinline__ u64 reduce64_40(u64 x, u64 q, u32 mu32) {
-    const u32 qe = __umulhi((u32)(x >> 32), mu32);
-    const u64 nq = 0 - q;  // x + qe (2^64 - q): two multiply-adds, no subtraction
-    return (u64)qe * (u32)nq + x + ((u64)(qe * (u32)(nq >> 32)) << 32);
+    u64 r;
+    asm("{\n\t.reg .u32 x0, x1, n0, n1, e, t0, t1;\n\t.reg .u64 t;\n\t"
+        "mov.b64 {x0, x1}, %1;\n\tmov.b64 {n0, n1}, %2;\n\t"
+        "mul.hi.u32 e, x1, %3;\n\tmad.wide.u32 t, e, n0, %1;\n\tmov.b64 {t0, t1}, t;\n\t"
+        "mad.lo.u32 t1, e, n1, t1;\n\tmov.b64 %0, {t0, t1};\n\t}" : "=l"(r) : "l"(x), "l"(0 - q), "r"(mu32));
+    return r;
 }
 
 // Sums of products without carries.  A carry chain costs an instruction per
@@ -185,7 +199,10 @@ struct Sum40 {
     // M + 2^12 P + 2^32 Q is below 2^64; its residue m < 3q < 2^42 leaves
     // L + add + 2^20 m below 2^63.
     __device__ __forceinline__ u64 value(u64 add, u64 q, u32 mu32) const {
-        const u64 m = reduce64_40(M + ((u64)P << 12) + ((u64)Q << 32), q, mu32);
+        u64 t;  // M + 2^12 P + 2^32 Q in 32-bit adds
+        asm("{\n\t.reg .u32 t0, t1, p0, p1;\n\tmov.b64 {t0, t1}, %2;\n\tshl.b32 p0, %1, 12;\n\tshr.u32 p1, %1, 20;\n\tadd.u32 p1, p1, %3;\n\t"
+            "add.cc.u32 t0, t0, p0;\n\taddc.u32 t1, t1, p1;\n\tmov.b64 %0, {t0, t1};\n\t}" : "=l"(t) : "r"(P), "l"(M), "r"(Q));
+        const u64 m = reduce64_40(t, q, mu32);
         return reduce64_40(L + add + (m << 20), q, mu32);
     }
 };
@@ -199,10 +216,9 @@ __device__ __forceinline__ void split20(u64 x, u32& l, u32& h) {  // x < 2^52
 struct Sum60 {
     u64 L = 0, M = 0, H = 0;
     __device__ __forceinline__ void mac(u32 d0, u32 d1, u32 k0, u32 k1) {
-        L += (u64)d0 * k0;
-        M += (u64)d0 * k1;
-        M += (u64)d1 * k0;
-        H += (u64)d1 * k1;
+        asm("mad.wide.u32 %0, %3, %5, %0;\n\tmad.wide.u32 %1, %3, %6, %1;\n\t"
+            "mad.wide.u32 %2, %4, %6, %2;\n\tmad.wide.u32 %1, %4, %5, %1;"
+            : "+l"(L), "+l"(M), "+l"(H) : "r"(d0), "r"(d1), "r"(k0), "r"(k1));
     }
     // L + 2^30 M + 2^60 H + add (add < 2^63) mod q, in [0, 5q)
     __device__ __forceinline__ u64 value(u64 add, const ModC& m) const {
