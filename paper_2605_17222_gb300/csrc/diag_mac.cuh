@@ -289,6 +289,12 @@ __device__ __forceinline__ void ws_compute(const WsCtx& c) {
     }
 }
 
+// The source run of phi_{n1 j} over run `run` (see the j table below).
+__device__ __forceinline__ u32 mid_run(u32 run, u32 g, u32 lr, u32 N) {
+    const u32 E = ((g * (2 * (__brev(run) >> (32 - lr)) + 1) - 1) >> 1) & (N - 1);
+    return __brev(E & ((1u << lr) - 1)) >> (32 - lr);
+}
+
 // Bytes of one stage: K3 diagonal blocks | beta digit runs | A run | key block (B run at j = 0).
 __host__ __device__ inline u32 ws_stage(bool packed, u32 k3, u32 beta, u32 beta_max) {
     const u32 kb = beta ? key_blk(packed, beta, beta_max) : 0;
@@ -341,7 +347,7 @@ __global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_c
         const u32 g = jj ? a.gal_mid[jj] : 1u;
         const u32 R = __brev(run) >> (32 - lr);
         const u32 E = ((g * (2 * R + 1) - 1) >> 1) & (N - 1);
-        jtab[jj] = (__brev(E & ((1u << lr) - 1)) >> (32 - lr)) | ((E >> lr) << 16) | ((g & 127u) << 24);
+        jtab[jj] = mid_run(run, g, lr, N) | ((E >> lr) << 16) | ((g & 127u) << 24);
     }
     if (l == 0) {
         for (u32 b = 0; b < ns; b++) {
@@ -358,12 +364,18 @@ __global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_c
 
     if (l >= BLK) {
         // ------------------------------------------------------------ producer warp
-        // One thread issues every copy, with straight-line code: a bulk copy
-        // takes its operands from uniform registers, so copies spread over the
-        // lanes of a warp are issued one lane at a time by a loop that moves
-        // each lane's operands there.
+        // Copies are issued by one thread, one after another.  A bulk copy takes
+        // its operands from uniform registers: spread over the lanes of a warp,
+        // copies are issued one lane at a time by a loop that moves each lane's
+        // operands there, and in a loop that one thread runs every operand is
+        // moved; only where the whole warp runs the loop and an elected lane
+        // issues are the addresses uniform to begin with.  That is what the wide
+        // limbs do, whose stages were bound by it (Set-A, ten copies a step: 1.03
+        // -> 0.93 ms, Set-B 0.65 -> 0.63).  The packed limbs at N = 2^16, bound
+        // by arithmetic, lost time to it (1.78 -> 1.90 ms) and keep one thread.
         u32 issued = 0;
-        if (l == BLK) {
+        const bool leader = PACKED ? l == BLK : elect_one();
+        if (!PACKED || leader) {
             const unsigned char* fsrc[K3];  // the next step's diagonal blocks
 #pragma unroll
             for (int kk = 0; kk < K3; kk++) {
@@ -375,44 +387,54 @@ __global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_c
             const size_t koff = m.koff + (size_t)run * key_blk(packed, a.beta_max, a.beta_max);
             const u32 group = a.slots * BLK;  // words from one block's group of slots to the next
             const size_t ox = bidx * a.bs_x + (size_t)t * (N / BLK) * group;
-            u32 sidx = 0, phase = 1, i = 0, j = 0;
+            u32 sidx = 0, phase = 1, i = 0, j = 0, srun = run;
             for (u32 it = 0; it < n1n2; it++) {
                 // every compute warp has read step it - ns, or giving up
-                if (it >= ns && !mbar_wait_abortable(&empty_bar[sidx], phase, DM_WAIT_NS, abort)) {
-                    *abort = 1u;
-                    break;
+                if (it >= ns) {
+                    bool ok = mbar_wait_abortable(&empty_bar[sidx], phase, DM_WAIT_NS, abort);
+                    if (!PACKED) ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) {
+                        *abort = 1u;
+                        break;
+                    }
                 }
                 issued = it + 1;
                 if (it != a.starve_step) {  // test hook: this step is never issued
                     const bool copy_a = i > 0 || !a.lift0 || lift_limb;
                     unsigned char* st = smem + sidx * stage;
                     u64* bar = &full_bar[sidx];
-                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     const u32 xb = (beta + (copy_a ? 1 : 0)) * RB;  // digits and A
-                    mbar_expect_tx(bar, k_count * fb + (j ? xb + kb : (copy_a ? 2 * RB : 0)));
-                    const u64* X = a.X[i] + ox + (size_t)(jtab[j] & 0xFFFFu) * group;
+                    const u64* X = a.X[i] + ox + (size_t)(PACKED ? jtab[j] & 0xFFFFu : srun) * group;
+                    const u64* B = (i || !a.lift0 ? a.B[i] + bidx * a.bs_b : a.c1[bidx]) + tN + (size_t)run * BLK;
+                    const unsigned char* K = a.keys[j] + koff;
+                    if (PACKED || leader) {
+                        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                        mbar_expect_tx(bar, k_count * fb + (j ? xb + kb : (copy_a ? 2 * RB : 0)));
 #pragma unroll
-                    for (int kk = 0; kk < K3; kk++)
-                        if (kk < (int)k_count) tma_load_1d(st + kk * fb, fsrc[kk], fb, bar);
-                    if (j) {
-                        tma_load_1d(st + off_dig, X, xb, bar);
-                        tma_load_1d(st + off_key, a.keys[j] + koff, kb, bar);
-                    } else if (copy_a) {
-                        tma_load_1d(st + off_a, X + group - BLK, RB, bar);
-                        const u64* B = i || !a.lift0 ? a.B[i] + bidx * a.bs_b : a.c1[bidx];
-                        tma_load_1d(st + off_key, B + tN + (size_t)run * BLK, RB, bar);
+                        for (int kk = 0; kk < K3; kk++)
+                            if (kk < (int)k_count) tma_load_1d(st + kk * fb, fsrc[kk], fb, bar);
+                        if (j) {
+                            tma_load_1d(st + off_dig, X, xb, bar);
+                            tma_load_1d(st + off_key, K, kb, bar);
+                        } else if (copy_a) {
+                            tma_load_1d(st + off_a, X + group - BLK, RB, bar);
+                            tma_load_1d(st + off_key, B, RB, bar);
+                        }
                     }
                 }
 #pragma unroll
                 for (int kk = 0; kk < K3; kk++) fsrc[kk] += a.diag_stride;
                 if (++sidx == ns) sidx = 0, phase ^= 1;
-                if (++i == n1) i = 0, j++;
+                if (++i == n1) {
+                    i = 0;
+                    if (++j < n2 && !PACKED) srun = mid_run(run, a.gal_mid[j], lr, N);
+                }
             }
         }
         __syncwarp();
         nbar_sync(1, WS_THREADS);  // every thread of the CTA reaches this once
         if (join && blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) pdl_wait();
-        if (*abort && l == BLK) {
+        if (*abort && leader) {
             // drain: the last phase issued into each stage (the earlier ones completed and were consumed)
             for (u32 it = issued > ns ? issued - ns : 0; it < issued; it++)
                 if (it != a.starve_step) mbar_wait_bounded(&full_bar[it % ns], (it / ns) & 1);

@@ -48,6 +48,12 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, u32 byte
         : "memory");
 }
 
+// One lane of a converged warp, known to the compiler as one.
+__device__ __forceinline__ bool elect_one() {
+    u32 p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void nbar_sync(u32 id, u32 count) {
     asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(count) : "memory");
 }
