@@ -31,7 +31,7 @@ namespace {
 // WS_MAX_STAGES; the packed limbs' stages are a quarter smaller, so they get
 // more).
 //
-// At the N = 2^16 (1,64,4) split, 10.3 GB of keys and diagonals: 1.78 ms (2.45
+// At the N = 2^16 (1,64,4) split, 10.3 GB of keys and diagonals: 1.74 ms (2.45
 // before: unpacked, 17 copies per step issued from the lanes of a warp,
 // 96-bit carry chains).  The copies alone take 1.13 ms for the 23 packed limbs
 // (6.7 TB/s), the arithmetic alone 1.2; the multiplier pipe is about 70% busy.
@@ -145,8 +145,10 @@ struct WsCtx {
 // A step is one serial chain per warp, and registers allow three or four warps
 // per scheduler, so its latency is what counts: the loop body has no branch
 // (BETA is exact, outer indices past k_count compute on stale words that are
-// never stored), so that every shared-memory load of a step is issued before
-// its arithmetic.
+// never stored), so that the middle layer's shared-memory loads are issued
+// together.  The diagonal words are read after its products, whose registers
+// they then take ((1,64,4) 1.78 -> 1.74 ms, Set-B 0.62 -> 0.58), but for the wide
+// limbs with one digit, which have registers to spare (Set-A 0.92, 0.96 late).
 template <int K3, int BETA, int CLS>
 __device__ __forceinline__ void ws_compute(const WsCtx& c) {
     constexpr u32 FULLM = 0xffffffffu;
@@ -243,8 +245,6 @@ __device__ __forceinline__ void ws_compute(const WsCtx& c) {
                     k[b] = kp[b * BLK];
                     if (!(b & 1)) w[b / 2] = hp[b / 2];
                 }
-                load_f(st);
-                release();
                 Sum40 s0, s1;
 #pragma unroll
                 for (int b = 0; b < BETA; b++) {
@@ -253,6 +253,8 @@ __device__ __forceinline__ void ws_compute(const WsCtx& c) {
                     s0.mac(dl, dh, k[b].x, (w[b / 2] >> (16 * (b & 1))) & 0xFFu);
                     s1.mac(dl, dh, k[b].y, (w[b / 2] >> (16 * (b & 1) + 8)) & 0xFFu);
                 }
+                load_f(st);
+                release();
                 av = s0.value(x, q, mu32);
                 bv = s1.value(0, q, mu32);
             } else {
@@ -260,8 +262,10 @@ __device__ __forceinline__ void ws_compute(const WsCtx& c) {
                 ulonglong2 k[BETA];
 #pragma unroll
                 for (int b = 0; b < BETA; b++) k[b] = kp[b * BLK];
-                load_f(st);
-                release();
+                if constexpr (BETA == 1) {
+                    load_f(st);
+                    release();
+                }
                 Sum60 s0, s1;
 #pragma unroll
                 for (int b = 0; b < BETA; b++) {
@@ -271,6 +275,10 @@ __device__ __forceinline__ void ws_compute(const WsCtx& c) {
                     s0.mac(dl, dh, kl, kh);
                     split30(k[b].y, kl, kh);
                     s1.mac(dl, dh, kl, kh);
+                }
+                if constexpr (BETA > 1) {
+                    load_f(st);
+                    release();
                 }
                 av = s0.value(x, m);
                 bv = s1.value(0, m);
