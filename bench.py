@@ -250,6 +250,14 @@ def lt_compulsory_bytes(split, level: int, k: int, beta: int, n_diag: int, N: in
     return 8 * N * (n_diag * ext + keys * 2 * beta * ext + 2 * level + 2 * (level - 1))
 
 
+def stored_ratio(ps, level: int, p_limbs: bool = True) -> float:
+    """Bytes the library stores a key or diagonal limb in (5 a word for moduli
+    between 2^32 and 2^40, else 8), over 8 bytes a word, averaged over the
+    limbs of the basis: the byte models above count 8-byte words."""
+    mods = list(ps.q[:level]) + (list(ps.p) if p_limbs else [])
+    return sum(5 if 2 ** 32 < m < 2 ** 40 else 8 for m in mods) / (8.0 * len(mods))
+
+
 def source_digest(paths) -> str:
     h = hashlib.sha256()
     for p in paths:
@@ -518,14 +526,19 @@ def run_ours(args, dist: Dist):
     b_lt, n_lt = algorithmic_bytes_for(algo, dominant, split3, LEVEL, ps.k, beta, D, ps.n, dh_sched == "fused")
     roof = None
     if b_lt and dom_n:
-        per_launch = b_lt / n_lt
+        b_lt *= stored_ratio(ps, LEVEL, not (algo == "bsgs" and dominant == "diag_mac"))
+        per_launch = b_lt * args.steps / dom_n
         avg_s = dom_ms / dom_n / 1e3
         ach = per_launch / avg_s / 1e9
         roof = {"kernel": dominant, "bound": "hbm", "achieved": round(ach, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(ach / peak, 4), "traffic": ncu_traffic(dominant),
                 "algorithmic_bytes_per_launch": int(per_launch), "avg_launch_ms": round(avg_s * 1e3, 4),
                 "peak_source": f"{peak_src} HBM copy bandwidth"}
-    lt_bytes = lt_compulsory_bytes(split3, LEVEL, ps.k, beta, D, ps.n) if algo in ("th", "dh") else None
+    lt_bytes = None
+    if algo in ("th", "dh"):  # ciphertexts at 8 bytes a word
+        ct_bytes = 8 * ps.n * (2 * LEVEL + 2 * (LEVEL - 1))
+        lt_bytes = int((lt_compulsory_bytes(split3, LEVEL, ps.k, beta, D, ps.n) - ct_bytes) * stored_ratio(ps, LEVEL)
+                       + ct_bytes)
     result = {
         "metric": METRIC, "value": round(value, 3), "unit": "LT/s", "n_gpus": dist.world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(max_ms / args.steps, 4),
@@ -651,7 +664,7 @@ def run_batched(args, dist: Dist):
         beta = g.beta(lv)
         ext = lv + ps.k
         keys = (sp[0] - 1) + (sp[1] - 1) + (sp[2] - 1)
-        comp += limb * (D * ext + keys * 2 * beta * ext)
+        comp += int(limb * (D * ext + keys * 2 * beta * ext) * stored_ratio(ps, lv))
     comp += sum(limb * (2 * lv + 2 * (lv - 1)) for lv in levels)
     peak = measured_peaks().get("hbm_gbs", 6800.0)
     val = dist.world * n_ct * steps / (ms_graph / 1e3)
@@ -853,7 +866,7 @@ def run_paper_shape(args, dist: Dist):
     limb = 8 * ps.n
     ext = lvl + ps.k
     keys = split[0] + split[1] + split[2] - 3
-    comp = limb * (Dn * ext + keys * 2 * g.beta(lvl) * ext + 2 * lvl + 2 * (lvl - 1))
+    comp = int(limb * (Dn * ext + keys * 2 * g.beta(lvl) * ext) * stored_ratio(ps, lvl)) + limb * (4 * lvl - 2)
     peak = measured_peaks().get("hbm_gbs", 6800.0)
     ms = total / steps
     return {
@@ -1009,7 +1022,7 @@ def run_chain(args, dist: Dist):
         amounts = [(off0 + stride * sp[0] * sp[1] * kk) % (N // 2) for kk in range(sp[2])]
         b, n = algorithmic_bytes(dominant, sp, lvl0 - i, ps.k, g.beta(lvl0 - i), Dn, N,
                                  outer_rotated=sum(1 for a in amounts if a))
-        per_chain += b
+        per_chain += b * stored_ratio(ps, lvl0 - i)
         per_chain_launches += n
     ach = per_chain * steps / (dom_ms / 1e3) / 1e9 if dom_ms else None
     unit = "CoeffToSlot/s" if kind == "cts" else "SlotToCoeff/s"
