@@ -627,8 +627,7 @@ DiagMacArgs dm_base(ckks_ctx* C, u32 level, bool with_p, const ckks_diags* f, u3
     a.beta = C->beta(level);
     a.beta_max = C->beta_max;
     a.log_n = C->log_n;
-    if (a.ext > (u32)DM_MAX_LIMBS) fail(CKKS_EINVAL, "more than 256 limbs in the extended basis");
-    for (int wide = 0; wide < 2; wide++)
+    for (int wide = 0; wide < 2 && a.ext <= (u32)DM_MAX_LIMBS; wide++)
         for (u32 t = 0, n = wide ? a.n_packed : 0; t < a.ext; t++)
             if (packed_q(C->mods[C->gmod(level, t)]) == !wide) {
                 a.limbs[n++] = (unsigned char)t;

@@ -243,7 +243,8 @@ struct DiagMacArgs {
     // Tile (0 = default): outer indices per CTA, a power of two below the
     // next power of two >= n3, at most 8.  Results do not depend on it.
     u32 tile_k3;
-    // the limbs t < ext: the packed_q ones, then the wide ones
+    // the limbs t < ext: the packed_q ones, then the wide ones (a basis of more
+    // than DM_MAX_LIMBS runs the plain kernel over every limb)
     u32 n_packed;
     unsigned char limbs[DM_MAX_LIMBS];
     // Batch of ciphertexts sharing the diagonals and keys: ciphertext b uses

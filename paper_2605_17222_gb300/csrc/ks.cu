@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_diag_mac(const __grid_constant__
     const u32 bidx = blockIdx.x % a.batch;
     const u32 s = (blockIdx.x / a.batch) * THREADS + threadIdx.x;
     const size_t ox = bidx * a.bs_x, ob = bidx * a.bs_b, ou = bidx * a.bs_u;
-    const u32 t = a.limbs[l0 + blockIdx.y];
+    const u32 t = a.ext <= (u32)DM_MAX_LIMBS ? a.limbs[l0 + blockIdx.y] : blockIdx.y;
     if (s >= N) return;
     const u32 k_first = blockIdx.z * K3;
     const u32 k_count = min((u32)K3, a.n3 - k_first);
@@ -473,6 +473,11 @@ void launch_diag_mac(const DiagMacArgs& a, cudaStream_t st) {
         count_launch();
     };
     auto both = [&](auto k3c) {
+        if (a.ext > (u32)DM_MAX_LIMBS) {
+            launch(false, k_diag_mac<decltype(k3c)::value>, grid, THREADS, 0, st, a, 0u);
+            count_launch();
+            return;
+        }
         run(k3c, std::false_type{}, false);
         run(k3c, std::true_type{}, a.n_packed < a.ext);
     };

@@ -103,18 +103,6 @@ __device__ __forceinline__ void mac96(U96& acc, u64 a, u64 b) {
         : "l"(a), "l"(b));
 }
 
-__device__ __forceinline__ void add96(U96& acc, u64 v) {
-    asm("{\n\t.reg .u32 w0, w1, v0, v1;\n\t"
-        "mov.b64 {w0, w1}, %0;\n\t"
-        "mov.b64 {v0, v1}, %2;\n\t"
-        "add.cc.u32 w0, w0, v0;\n\t"
-        "addc.cc.u32 w1, w1, v1;\n\t"
-        "addc.u32 %1, %1, 0;\n\t"
-        "mov.b64 %0, {w0, w1};\n\t}"
-        : "+l"(acc.lo), "+r"(acc.hi)
-        : "l"(v));
-}
-
 __device__ __forceinline__ void add128(U128& acc, u64 v) {
     asm("add.cc.u64 %0, %0, %2;\n\t"
         "addc.u64 %1, %1, 0;"

@@ -176,12 +176,6 @@ __device__ __forceinline__ void ct_bfly_w(u64& a, u64& b, u64 w, u64 ws, u64 q) 
     a = x + v;
     b = x - v + q2;
 }
-__device__ __forceinline__ void ct_bfly(u64& a, u64& b, const ulonglong2* tab, u32 idx, u64 q) {
-    u64 w, ws;
-    tw_at(tab, idx, w, ws);
-    ct_bfly_w(a, b, w, ws, q);
-}
-
 // [0, 4q) -> [0, q)
 __device__ __forceinline__ u64 canon4(u64 x, u64 q) {
     x = x >= 2 * q ? x - 2 * q : x;
