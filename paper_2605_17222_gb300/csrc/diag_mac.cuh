@@ -3,6 +3,7 @@
 // the instances compile in parallel.
 #pragma once
 #include "kernels.h"
+#include "ks_products.cuh"
 #include "mbar.cuh"
 
 #include <algorithm>
@@ -46,6 +47,11 @@ namespace {
 // pending -- sets *err, and the CTA writes no output.
 constexpr u32 WS_THREADS = BLK + 32;
 constexpr u32 WS_MAX_STAGES = 6;
+// BETA of the instance for more than eight digits: a loop over groups of four
+// digits from the stage, two CTAs per SM, or one if two stages need it.  Sixteen
+// digits at N = 2^15, the (1,8,4) split: 229 us, and 286 at (2,4,8); the plain
+// kernel takes 623 and 793 with branches between a group's loads.
+constexpr int WS_ANY = 9;
 
 // Sums of v * f, v a middle-layer word and f a diagonal word, per class of
 // limb (chosen once per CTA).  TERMS products fit between two reductions.
@@ -232,6 +238,14 @@ __device__ __forceinline__ void ws_compute(const WsCtx& c) {
             const unsigned char* st = c.smem + sidx * c.stage;
             const u64 x = zero ? 0 : ((const u64*)(st + c.off_a))[pm];
             const u64* dg = (const u64*)(st + K3 * FB) + pm;
+            if constexpr (BETA == WS_ANY) {
+                u64 av = x, bv = 0;
+                ks_products<CLS == C40>(m, dg, BLK, st + off_key, l, a.beta, a.beta_max, av, bv);
+                load_f(st);
+                release();
+                outer(av, bv);
+                continue;
+            }
             u64 d[BETA], av, bv;
 #pragma unroll
             for (int b = 0; b < BETA; b++) d[b] = dg[b * BLK];
@@ -338,7 +352,7 @@ __global__ void __launch_bounds__(WS_THREADS, MINB) k_diag_mac_ws(const __grid_c
     constexpr bool packed = PACKED;
     const size_t tN = (size_t)t * N;
     const u32 n1 = a.n1, n2 = a.n2, n1n2 = n1 * n2;
-    constexpr u32 beta = BETA;  // a.beta, or 0 without a middle layer
+    const u32 beta = BETA == WS_ANY ? a.beta : BETA;  // a.beta, or 0 without a middle layer
     const u32 fb = diag_blk(packed);
     const u32 kb = beta ? key_blk(packed, beta, a.beta_max) : 0;
     const u32 off_dig = K3 * fb, off_a = off_dig + beta * RB, off_key = off_a + RB;
@@ -474,13 +488,21 @@ constexpr u32 SM_SMEM = 227 * 1024;
 
 template <int K3, int BETA, int MINB, bool PACKED>
 bool try_ws(const DiagMacArgs& a, bool join, cudaStream_t st) {
-    constexpr u32 beta = BETA;
+    const u32 beta = BETA == WS_ANY ? a.beta : BETA;
     const u32 N = 1u << a.log_n;
-    // one CTA's share, less the 1 KB that the system takes per CTA and the static barriers
-    const u32 tab = (4 * a.n2 + 15) & ~15u, share = SM_SMEM / MINB - 1024 - 256;
-    if (tab >= share) return false;
-    const u32 ring = (share - tab) & ~127u;
-    if (ring < 2 * ws_stage(PACKED, K3, beta, a.beta_max)) return false;
+    // one CTA's share, less the 1 KB that the system takes per CTA and the static
+    // barriers; past eight digits a CTA may need all of it for two stages
+    const u32 tab = (4 * a.n2 + 15) & ~15u;
+    constexpr int MIN_CTAS = BETA == WS_ANY ? 1 : MINB;
+    u32 ring = 0;
+    for (int ctas = MINB; ctas >= MIN_CTAS; ctas--) {
+        const u32 share = SM_SMEM / ctas - 1024 - 256;
+        if (tab >= share) continue;
+        ring = (share - tab) & ~127u;
+        if (ring >= 2 * ws_stage(PACKED, K3, beta, a.beta_max)) break;
+        ring = 0;
+    }
+    if (!ring) return false;
     static std::atomic<uint64_t> attr_set{0}, attr_bad{0};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
@@ -491,7 +513,7 @@ bool try_ws(const DiagMacArgs& a, bool join, cudaStream_t st) {
     if (attr_bad.load(std::memory_order_relaxed) & bit) return false;
     if (!(attr_set.load(std::memory_order_acquire) & bit)) {
         if (cudaFuncSetAttribute(k_diag_mac_ws<K3, BETA, MINB, PACKED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(SM_SMEM / MINB - 1024 - 256)) != cudaSuccess) {
+                                 (int)(SM_SMEM / MIN_CTAS - 1024 - 256)) != cudaSuccess) {
             cudaGetLastError();
             attr_bad.fetch_or(bit, std::memory_order_relaxed);
             return false;
@@ -524,7 +546,7 @@ bool launch_ws(const DiagMacArgs& a, bool join, cudaStream_t st) {
         case 6: return try_ws<K3, 6, MINB, PACKED>(a, join, st);
         case 7: return try_ws<K3, 7, MINB, PACKED>(a, join, st);
         case 8: return try_ws<K3, 8, MINB, PACKED>(a, join, st);
-        default: return false;
+        default: return try_ws<K3, WS_ANY, 2, PACKED>(a, join, st);
     }
 }
 

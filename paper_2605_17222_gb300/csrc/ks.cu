@@ -15,6 +15,7 @@
 // Sum60, Outer3) and are reduced once (PE modes CWPM-ACC / CM-ACC of Sec. V,
 // done lazily).
 #include "kernels.h"
+#include "ks_products.cuh"
 #include "mbar.cuh"
 
 #include <algorithm>
@@ -32,44 +33,6 @@ __device__ __forceinline__ u64 diag_at(const unsigned char* limb, u32 s, bool pa
     const unsigned char* b = limb + (size_t)(s / BLK) * (BLK * 5);
     const u32 l = s % BLK;
     return ((const u32*)b)[l] | (u64)b[BLK * 4 + l] << 32;
-}
-
-// v_c += sum_b d_b k_{b,c} for one position (l of a key block K), b < beta, the
-// result in [0, 3q) (packed) or [0, 5q); four digits between two reductions.
-__device__ __forceinline__ void ks_products(const ModC& m, bool packed, const u64* D, size_t dstep,
-                                            const unsigned char* K, u32 l, u32 beta, u32 beta_max, u64& v0, u64& v1) {
-    constexpr u32 G = 4;
-    const u32 hb = key_hi(beta_max);
-    const uint2* lp = (const uint2*)(K + BLK * hb) + l;
-    const ulonglong2* kp = (const ulonglong2*)K + l;
-    for (u32 b0 = 0; b0 < beta; b0 += G) {
-        Sum40 s0, s1;
-        Sum60 t0, t1;
-#pragma unroll
-        for (u32 j = 0; j < G; j++) {
-            const u32 b = b0 + j;
-            if (b >= beta) break;
-            const u64 d = D[b * dstep];
-            u32 dl, dh;
-            if (packed) {
-                const uint2 k = lp[b * BLK];
-                const unsigned char* h = K + l * hb + 2 * b;
-                split20(d, dl, dh);
-                s0.mac(dl, dh, k.x, h[0]);
-                s1.mac(dl, dh, k.y, h[1]);
-            } else {
-                const ulonglong2 k = kp[b * BLK];
-                u32 kl, kh;
-                split30(d, dl, dh);
-                split30(k.x, kl, kh);
-                t0.mac(dl, dh, kl, kh);
-                split30(k.y, kl, kh);
-                t1.mac(dl, dh, kl, kh);
-            }
-        }
-        v0 = packed ? s0.value(v0, m.q, (u32)m.mu_hi) : t0.value(v0, m);
-        v1 = packed ? s1.value(v1, m.q, (u32)m.mu_hi) : t1.value(v1, m);
-    }
 }
 
 // ------------------------------------------------------------------ K4
@@ -217,7 +180,9 @@ __global__ void __launch_bounds__(BLK, 8) k_ks_ws(const __grid_constant__ KsArgs
     }
 }
 
-// Any number of digits, operands straight from global memory (more than eight digits).
+// Any number of digits, operands straight from global memory: more than eight
+// digits, or unaligned ones.  Sixteen digits at N = 2^15, the seven products of the
+// (1,8,4) split: 119 us.
 __global__ void __launch_bounds__(BLK) k_ks_any(const __grid_constant__ KsArgs a) {
     const u32 first = a.sum ? 0 : blockIdx.x % a.count, last = a.sum ? a.count : first + 1;
     const u32 run = a.sum ? blockIdx.x : blockIdx.x / a.count;
@@ -233,8 +198,9 @@ __global__ void __launch_bounds__(BLK) k_ks_any(const __grid_constant__ KsArgs a
         const KsItem& E = a.e[e];
         const u32 src = E.gal ? auto_src(p.s, E.gal, a.log_n) : p.s;
         v0 += ks_x0(a, E, p, src, m.q);
-        ks_products(m, packed, E.digits + p.t * a.dl.limb + (src / BLK) * a.dl.blk + src % BLK, a.dl.dig, E.key + koff,
-                    threadIdx.x, a.beta, a.beta_max, v0, v1);
+        const u64* D = E.digits + p.t * a.dl.limb + (src / BLK) * a.dl.blk + src % BLK;
+        if (packed) ks_products<true>(m, D, a.dl.dig, E.key + koff, threadIdx.x, a.beta, a.beta_max, v0, v1);
+        else ks_products<false>(m, D, a.dl.dig, E.key + koff, threadIdx.x, a.beta, a.beta_max, v0, v1);
     }
     if (a.sum) a.e[0].out0[o] = canon8(v0, m.q), a.e[0].out1[o] = canon8(v1, m.q);
     else ks_store(a, a.e[first], p, v0, v1, m.q);
@@ -253,7 +219,7 @@ __global__ void __launch_bounds__(BLK) k_ks_any(const __grid_constant__ KsArgs a
 // method n1 = 1, BSGS n2 = 1 over Q only.
 //
 // This plain form reads its operands straight from global memory; it runs the
-// shapes whose stages do not fit the staged kernel below (more than eight digits).
+// shapes whose stages do not fit the staged kernel (about forty digits) and unaligned operands.
 template <int K3>
 __global__ void __launch_bounds__(THREADS, 2) k_diag_mac(const __grid_constant__ DiagMacArgs a, u32 l0) {
     const u32 N = 1u << a.log_n;
@@ -303,7 +269,8 @@ __global__ void __launch_bounds__(THREADS, 2) k_diag_mac(const __grid_constant__
                 if (!lifted) bv = (a.B[i] + ob)[tN + s];
                 else if (lift_limb) bv = mul_shoup(a.c1[bidx][tN + s], lc, lsh, m.q);
             } else {
-                ks_products(m, packed, X, BLK, a.keys[j] + koff, s % BLK, a.beta, a.beta_max, av, bv);
+                if (packed) ks_products<true>(m, X, BLK, a.keys[j] + koff, s % BLK, a.beta, a.beta_max, av, bv);
+                else ks_products<false>(m, X, BLK, a.keys[j] + koff, s % BLK, a.beta, a.beta_max, av, bv);
             }
 #pragma unroll
             for (int kk = 0; kk < K3; kk++) {

@@ -57,6 +57,24 @@ def test_mixed_moduli_lt(dnum, level, D, split, algo, offset0):
         g.close()
 
 
+@pytest.mark.parametrize("copies,level,split", [
+    (2, 18, (1, 3, 1)),   # 18 digits: groups of four and a rest of two; one outer index
+    (2, 13, (2, 2, 2)),   # a rest of one
+    (2, 12, (1, 4, 3)),   # no rest; a tile of four with an idle index
+    (2, 10, (1, 2, 9)),   # eight outer indices and one more
+    (4, 36, (1, 2, 8)),   # stages too large for the wide limbs: the plain kernel for them
+])
+def test_more_than_eight_digits(monkeypatch, copies, level, split):
+    monkeypatch.setitem(globals(), "Q_BITS", Q_BITS * copies)
+    g, f, ct, want = problem(9 * copies, level, int(np.prod(split)), split, "th")
+    try:
+        got, _ = g.lt_eval(g.ct_from_host(ct), f, "th", split)
+        assert_same(got.numpy(), want, f"{split} {level} digits")
+        g.device_status()
+    finally:
+        g.close()
+
+
 def test_words_beyond_the_modulus_are_taken_as_residues():
     """Diagonals written in pieces, with words in [q, 2q), give the same result as their residues."""
     import torch
