@@ -342,6 +342,16 @@ struct Arena {
         blocks.push_back(p);
         return (u64*)p;
     }
+    // The same, or null where the device has not that much memory left.
+    u64* limbs_or_null(size_t n) {
+        try {
+            return limbs(n);
+        } catch (const Fail& e) {
+            if (e.st != CKKS_ENOMEM) throw;
+            cudaGetLastError();  // not left for a later status check
+            return nullptr;
+        }
+    }
     ~Arena() {
         for (void* p : blocks) cudaFreeAsync(p, st);
     }
@@ -888,6 +898,12 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
 // rotated c1 and two ModDowns), products over Q, plain rescale at the end.
 // The baby steps are independent of one another, and so are the giant steps:
 // each layer runs in chunks of rotations, every step of a chunk one launch.
+// A chunk's whole scratch, what its rotations leave for the sums included, is
+// at most BSGS_SCRATCH bytes (one rotation at least), and where the device has
+// not even that left, the chunks are halved until they fit: one rotation at a
+// time takes no more than a sequence of ckks_ks_inner and ckks_moddown does.
+constexpr size_t BSGS_SCRATCH = size_t(512) << 20;
+
 void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 n2, cudaStream_t st, u32 tile = 0) {
     const u32 N = C->N, K = C->K, ext = level + K, beta = C->beta(level);
     const int64_t s = f->stride;
@@ -896,20 +912,30 @@ void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u3
     struct Rot {
         const u64 *c0, *c1;
         int64_t r;
-        u64 *o0, *o1;  // T0 = ModDown of the first output and the rotated second component
+        u64 *o0, *o1;  // a baby step's rotated pair; null for a giant step, which is summed chunk by chunk
     };
-    // limbs of scratch per rotation: digits, the two products, ModDown and Decompose sources; a
-    // chunk takes at most 512 MB of it (one rotation at least)
-    const size_t per = (size_t)beta * ext + 2 * ext + std::max<size_t>(level, 2 * K);
-    const u32 widest = std::max<u32>(1, std::max<u32>(n1 - 1, (u32)ol.rotated.size()));
-    const u32 chunk = (u32)std::min<size_t>(widest, std::max<size_t>(1, (size_t(512) << 20) / (per * N * 8)));
-    u64* D = ar.limbs((size_t)chunk * beta * ext);
-    u64* P = ar.limbs((size_t)chunk * 2 * ext);
-    u64* Y = ar.limbs(std::max<size_t>((size_t)chunk * std::max(level, 2 * K), 4));
-    // ModDown(<Decompose(phi_r(c1)), swk_r>) of every rotation into (o0, o1)
-    auto switch_keys = [&](const std::vector<Rot>& rots) {
-        for (size_t b = 0; b < rots.size(); b += chunk) {
-            const u32 n = (u32)std::min<size_t>(chunk, rots.size() - b);
+    // limbs of scratch per rotation: the digits, whose place the ModDowns' outputs take once the
+    // products are formed; the two products; ModDown and Decompose sources
+    const size_t dig = std::max<size_t>((size_t)beta * ext, 2 * level), src = std::max<size_t>(level, 2 * K);
+    const size_t per = dig + 2 * ext + src;
+    struct Part {
+        u64 *D, *P, *Y;  // [chunk] of digits, products, sources
+        u32 chunk;
+    };
+    auto part = [&](size_t rots) {
+        u32 chunk = (u32)std::min(std::max<size_t>(rots, 1), std::max<size_t>(1, BSGS_SCRATCH / (per * N * 8)));
+        u64* D;
+        while (!(D = ar.limbs_or_null(chunk * per))) {
+            if (chunk == 1) fail(CKKS_ENOMEM, "no device memory for one rotation");
+            chunk = (chunk + 1) / 2;
+        }
+        return Part{D, D + chunk * dig * N, D + chunk * (dig + 2 * ext) * N, chunk};
+    };
+    // Per chunk of rotations: ModDown(<Decompose(phi_r(c1)), swk_r>), a baby step's second component into o1,
+    // then take(the chunk's first rotation, their number, the ModDowns' outputs in pairs).
+    auto switch_keys = [&](const Part& W, const std::vector<Rot>& rots, auto&& take) {
+        for (size_t b = 0; b < rots.size(); b += W.chunk) {
+            const u32 n = (u32)std::min<size_t>(W.chunk, rots.size() - b);
             std::vector<const u64*> cs, xs;
             std::vector<u32> gals;
             std::vector<u64*> ds, outs;
@@ -918,18 +944,19 @@ void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u3
                 const Rot& R = rots[b + i];
                 cs.push_back(R.c1);
                 gals.push_back(C->galois(R.r));
-                ds.push_back(D + (size_t)i * beta * ext * N);
-                u64 *x0 = P + (size_t)i * 2 * ext * N, *x1 = x0 + (size_t)ext * N;
+                ds.push_back(W.D + i * dig * N);
+                u64 *x0 = W.P + (size_t)i * 2 * ext * N, *x1 = x0 + (size_t)ext * N;
                 es.push_back(KsItem{ds[i], key_of(C, R.r), nullptr, x0, x1, 0, 0});
                 xs.push_back(x0);
                 xs.push_back(x1);
-                outs.push_back(R.o0);
-                outs.push_back(R.o1);
+                outs.push_back(ds[i]);
+                outs.push_back(R.o1 ? R.o1 : ds[i] + (size_t)level * N);
             }
-            op_decompose_batch(C, level, cs, gals, ds, beta, Y, st);
+            op_decompose_batch(C, level, cs, gals, ds, beta, W.Y, st);
             KsArgs k = ks_base(C, level, beta, 0);
             op_ks_list(k, es, st);
-            op_moddown_batch(C, level, xs, outs, Y, st);
+            op_moddown_batch(C, level, xs, outs, W.Y, st);
+            take(rots.data() + b, n, outs);
         }
     };
     DiagMacArgs a = dm_base(C, level, false, f, tile);
@@ -939,19 +966,11 @@ void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u3
     a.slots = 1;
     a.X[0] = io.c0;
     a.B[0] = io.c1;
-    if (n1 > 1) {
-        std::vector<Rot> rots;
-        std::vector<AddJob> add;
-        for (u32 i = 1; i < n1; i++) {
-            u64 *t0 = ar.limbs(level), *c0 = ar.limbs(level), *c1 = ar.limbs(level);
-            rots.push_back(Rot{io.c0, io.c1, s * i, t0, c1});
-            a.X[i] = c0;
-            a.B[i] = c1;
-            for (u32 t = 0; t < level; t++)
-                add.push_back(AddJob{io.c0 + (size_t)t * N, t0 + (size_t)t * N, c0 + (size_t)t * N, t, C->galois(s * i)});
-        }
-        switch_keys(rots);
-        launch_add_gather((const ModC*)C->d_mods.p, add.data(), (int)add.size(), C->log_n, st);
+    std::vector<Rot> baby, giant;
+    for (u32 i = 1; i < n1; i++) {
+        baby.push_back(Rot{io.c0, io.c1, s * i, ar.limbs(level), ar.limbs(level)});
+        a.X[i] = baby.back().o0;
+        a.B[i] = baby.back().o1;
     }
     std::vector<u64*> V0(n2), V1(n2);
     for (u32 j = 0; j < n2; j++) {
@@ -961,27 +980,33 @@ void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u3
         a.U1[j] = V1[j];
         a.gal_diag[j] = ol.amount[j] ? C->galois(-ol.amount[j]) : 0;
     }
-    launch_diag_mac(a, st);
+    for (u32 j : ol.rotated) giant.push_back(Rot{V0[j], V1[j], ol.amount[j], nullptr, nullptr});
     u64* acc0 = ol.identity >= 0 ? V0[ol.identity] : ar.limbs(level);
     u64* acc1 = ol.identity >= 0 ? V1[ol.identity] : ar.limbs(level);
+    const Part W = part(std::max(baby.size(), giant.size()));  // last, so that it takes what is left
+    switch_keys(W, baby, [&](const Rot* R, u32 n, const std::vector<u64*>& outs) {
+        std::vector<AddJob> add;
+        for (u32 k = 0; k < n; k++)
+            for (u32 t = 0; t < level; t++)
+                add.push_back(AddJob{R[k].c0 + (size_t)t * N, outs[2 * k] + (size_t)t * N, R[k].o0 + (size_t)t * N, t,
+                                     C->galois(R[k].r)});
+        launch_add_gather((const ModC*)C->d_mods.p, add.data(), (int)add.size(), C->log_n, st);
+    });
+    launch_diag_mac(a, st);
     if (ol.identity < 0) {
         CK(cudaMemsetAsync(acc0, 0, (size_t)level * N * sizeof(u64), st));
         CK(cudaMemsetAsync(acc1, 0, (size_t)level * N * sizeof(u64), st));
     }
-    if (!ol.rotated.empty()) {
-        std::vector<Rot> rots;
-        for (u32 j : ol.rotated) rots.push_back(Rot{V0[j], V1[j], ol.amount[j], ar.limbs(level), ar.limbs(level)});
-        switch_keys(rots);
-        for (size_t b = 0; b < rots.size(); b += SUM_MAX) {
+    switch_keys(W, giant, [&](const Rot* R, u32 n, const std::vector<u64*>& outs) {
+        for (u32 k0 = 0; k0 < n; k0 += SUM_MAX) {
             SumArgs m;
             memset(&m, 0, sizeof(m));
-            m.count = (u32)std::min<size_t>(SUM_MAX, rots.size() - b);
+            m.count = std::min<u32>(SUM_MAX, n - k0);
             for (u32 k = 0; k < m.count; k++) {
-                const Rot& R = rots[b + k];
-                m.a[k] = R.c0;
-                m.b0[k] = R.o0;
-                m.b1[k] = R.o1;
-                m.gal[k] = C->galois(R.r);
+                m.a[k] = R[k0 + k].c0;
+                m.b0[k] = outs[2 * (k0 + k)];
+                m.b1[k] = outs[2 * (k0 + k) + 1];
+                m.gal[k] = C->galois(R[k0 + k].r);
             }
             m.acc0 = acc0;
             m.acc1 = acc1;
@@ -990,8 +1015,8 @@ void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u3
             m.log_n = C->log_n;
             launch_sum_gather(m, st);
         }
-    }
-    op_rescale_batch(C, level, {acc0, acc1}, {io.o0, io.o1}, Y, st);
+    });
+    op_rescale_batch(C, level, {acc0, acc1}, {io.o0, io.o1}, W.Y, st);
 }
 
 void validate_split(lt_algo algo, u32 D, const lt_split& sp) {
