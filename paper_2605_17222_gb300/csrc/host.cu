@@ -35,8 +35,9 @@ struct Fail {
 }
 
 void cuda_check(cudaError_t e, const char* what) {
-    if (e != cudaSuccess) fail(e == cudaErrorMemoryAllocation ? CKKS_ENOMEM : CKKS_ECUDA,
-                               std::string(what) + ": " + cudaGetErrorString(e));
+    if (e == cudaSuccess) return;
+    cudaGetLastError();  // reported here, and not once more by the next call's status check
+    fail(e == cudaErrorMemoryAllocation ? CKKS_ENOMEM : CKKS_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 #define CK(x) cuda_check((x), #x)
 
@@ -348,7 +349,6 @@ struct Arena {
             return limbs(n);
         } catch (const Fail& e) {
             if (e.st != CKKS_ENOMEM) throw;
-            cudaGetLastError();  // not left for a later status check
             return nullptr;
         }
     }
@@ -1410,24 +1410,30 @@ static void put_key(ckks_ctx* ctx, int32_t r, const uint64_t* src, size_t n_word
     if (n_words != ctx->key_words()) fail(CKKS_EINVAL, "key size must be beta_max*2*(L+k)*N words");
     CK(cudaSetDevice(ctx->device));
     const u32 rk = ctx->rotkey(r);
-    unsigned char* d;
     auto it = ctx->keys.find(rk);
-    if (it != ctx->keys.end()) d = it->second;
-    else d = (unsigned char*)ctx->dalloc(ctx->key_bytes / 8);
-    ctx->keys[rk] = d;
-    PackArgs p = pack_args(ctx, src, d);
-    if (kind == cudaMemcpyHostToDevice) {
-        u64* tmp = ctx->dalloc(n_words);
-        CK(cudaMemcpy(tmp, src, n_words * 8, kind));
-        p.in = tmp;
-        launch_pack_key(p, 0);
-        CK(cudaGetLastError());
-        CK(cudaDeviceSynchronize());
+    const bool replaced = it != ctx->keys.end();
+    unsigned char* d = replaced ? it->second : (unsigned char*)ctx->dalloc(ctx->key_bytes / 8);
+    u64* tmp = nullptr;
+    try {
+        PackArgs p = pack_args(ctx, src, d);
+        if (kind == cudaMemcpyHostToDevice) {
+            tmp = ctx->dalloc(n_words);
+            CK(cudaMemcpy(tmp, src, n_words * 8, kind));
+            p.in = tmp;
+            launch_pack_key(p, 0);
+            CK(cudaGetLastError());
+            CK(cudaDeviceSynchronize());
+            ctx->dfree(tmp, n_words);
+        } else {
+            launch_pack_key(p, st);
+            CK(cudaGetLastError());
+        }
+    } catch (...) {
         ctx->dfree(tmp, n_words);
-    } else {
-        launch_pack_key(p, st);
-        CK(cudaGetLastError());
+        if (!replaced) ctx->dfree((u64*)d, ctx->key_bytes / 8);
+        throw;
     }
+    ctx->keys[rk] = d;  // known from here on: a key whose upload failed stays unknown
 }
 
 ckks_status ckks_upload_rotation_key(ckks_ctx* ctx, int32_t r, const uint64_t* host, size_t n_words) {
