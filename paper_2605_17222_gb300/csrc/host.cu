@@ -1449,16 +1449,47 @@ int ckks_has_rotation_key(const ckks_ctx* ctx, int32_t r) {
     return ctx && ctx->keys.count(ctx->rotkey(r)) ? 1 : 0;
 }
 
+// Bytes of unpacked diagonals staged at a time (one diagonal at least).
+constexpr size_t STAGE_BYTES = size_t(256) << 20;
+static u32 stage_diags(const ckks_diags* f, u32 count) {
+    const size_t one = (size_t)(f->level + f->ctx->K) * f->ctx->N * 8;
+    return (u32)std::min<size_t>(count, std::max<size_t>(1, STAGE_BYTES / one));
+}
+
+// Whether a kernel on the context's device may read words at p.  Another
+// device's memory, the host's, or words at an odd byte are left to the copy
+// engine, which takes or refuses them.
+static bool kernel_readable(const ckks_ctx* ctx, const void* p) {
+    if ((uintptr_t)p % sizeof(u64)) return false;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == ctx->device);
+}
+
 // Packs diagonals [first, first + count) of f from words [count][level + k][N]
-// on the device, in stream order.
+// in stream order, straight from `dev` where a kernel can read it, else through
+// a staging buffer.
 static void pack_diags(const ckks_diags* f, u32 first, u32 count, const u64* dev, cudaStream_t st) {
     const ckks_ctx* ctx = f->ctx;
-    PackArgs p = pack_args(ctx, dev, f->d + (size_t)first * ctx->diag_bytes(f->level));
-    p.level = f->level;
-    p.p_base = ctx->q_bytes[f->level];
-    p.stride = ctx->diag_bytes(f->level);
-    launch_pack_diags(p, count, st);
-    CK(cudaGetLastError());
+    const size_t limbs = f->level + ctx->K;
+    const bool direct = kernel_readable(ctx, dev);
+    const u32 chunk = direct ? count : stage_diags(f, count);
+    Arena ar(st, ctx->N);
+    u64* tmp = direct ? nullptr : ar.limbs(limbs * chunk);
+    for (u32 d0 = 0; d0 < count; d0 += chunk) {
+        const u32 n = std::min(chunk, count - d0);
+        const u64* in = dev + limbs * ctx->N * d0;
+        if (!direct) CK(cudaMemcpyAsync(tmp, in, limbs * ctx->N * n * 8, cudaMemcpyDeviceToDevice, st));
+        PackArgs p = pack_args(ctx, direct ? in : tmp, f->d + (size_t)(first + d0) * ctx->diag_bytes(f->level));
+        p.level = f->level;
+        p.p_base = ctx->q_bytes[f->level];
+        p.stride = ctx->diag_bytes(f->level);
+        launch_pack_diags(p, n, st);
+        CK(cudaGetLastError());
+    }
 }
 
 static void put_diags(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, int32_t offset0, int32_t stride,
@@ -1483,9 +1514,9 @@ static void put_diags(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, int32_t 
         u64* tmp = nullptr;
         size_t tmp_words = 0;
         try {
-            if (kind == cudaMemcpyHostToDevice) {  // through a staging buffer of at most 256 MB, or one diagonal
+            if (kind == cudaMemcpyHostToDevice) {
                 const size_t per = (size_t)(level + ctx->K) * ctx->N;
-                const u32 chunk = (u32)std::min<size_t>(n_diag, std::max<size_t>(1, (size_t(256) << 20) / (per * 8)));
+                const u32 chunk = stage_diags(f.get(), n_diag);
                 tmp_words = per * chunk;
                 tmp = ctx->dalloc(tmp_words);
                 for (u32 d0 = 0; d0 < n_diag; d0 += chunk) {

@@ -1,4 +1,4 @@
-"""Uploads that fail leave nothing behind."""
+"""Uploads from any memory, beside a recording, and at the limits of memory; the ones that fail leave nothing behind."""
 import contextlib
 import ctypes
 
@@ -50,6 +50,54 @@ def test_a_key_whose_upload_failed_stays_unknown():
             assert g.bytes_in_use() == used
         g.upload_rotation_key(5, key)
         assert g.has_key(5)
+        g.device_status()
+    finally:
+        g.close()
+
+
+def diagonals(ps, D):
+    from paper_2605_17222_gb300 import synth
+    return np.ascontiguousarray(synth.uniform_mod(5, "f", ps.moduli, ps.n * D).reshape(len(ps.moduli), D, ps.n)
+                                .transpose(1, 0, 2))
+
+
+def lt_of(g, ps, f, ct=None):
+    """The LT of one fixed ciphertext, without rotations' keys but the ones of a window of four."""
+    from paper_2605_17222_gb300 import synth
+    for r in (1, 2, 3):
+        if not g.has_key(r):
+            k = np.broadcast_to(synth.uniform_mod(r, "k", ps.moduli, ps.n), (g.beta_max, 2, len(ps.moduli), ps.n))
+            g.upload_rotation_key(r, np.ascontiguousarray(k))
+    c = np.stack([synth.uniform_mod(7 + c, "ct", ps.q, ps.n) for c in range(2)])
+    return g.lt_eval(g.ct_from_host(c), f, "th", (1, 2, 2))[0].numpy()
+
+
+@pytest.mark.parametrize("where", ["pinned", "pageable", "half a word off"])
+def test_device_upload_from_other_memory(where):
+    """A pointer that is not this device's memory, or not at a word, goes to the copy engine and never to a
+    kernel: it is copied or refused.  Host memory stands for another GPU's."""
+    import torch
+
+    from paper_2605_17222_gb300 import binding, synth
+    ps = synth.param_set("toy")
+    g = binding.Context.from_params(ps)
+    f = diagonals(ps, 4)
+    try:
+        want = lt_of(g, ps, g.upload_diagonals(f))
+        src = torch.from_numpy(f.view(np.int64))
+        if where == "pinned":
+            src = src.pin_memory()
+        elif where != "pageable":
+            src = torch.cat([torch.zeros(1, dtype=torch.int32), src.view(torch.int32).flatten()]).cuda()[1:]
+            assert src.data_ptr() % 8 == 4
+        part = g.diags_create(4)
+        st = binding.lib().ckks_diags_write_device(part.handle, 0, 4, ctypes.c_void_p(src.data_ptr()), f.size,
+                                                   binding._stream(None))
+        torch.cuda.synchronize()
+        if st != 0:  # nothing of a refused call is left
+            assert where == "pageable"
+            g.diags_write(part, 0, binding.to_device(f))
+        assert np.array_equal(lt_of(g, ps, part), want)
         g.device_status()
     finally:
         g.close()
