@@ -1422,7 +1422,7 @@ static void put_key(ckks_ctx* ctx, int32_t r, const uint64_t* src, size_t n_word
             p.in = tmp;
             launch_pack_key(p, 0);
             CK(cudaGetLastError());
-            CK(cudaDeviceSynchronize());
+            CK(cudaStreamSynchronize(0));  // not the device: another thread may be recording a stream of it
             ctx->dfree(tmp, n_words);
         } else {
             launch_pack_key(p, st);
@@ -1524,7 +1524,7 @@ static void put_diags(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, int32_t 
                     CK(cudaMemcpy(tmp, host + per * d0, per * n * 8, kind));
                     pack_diags(f.get(), d0, n, tmp, 0);
                 }
-                CK(cudaDeviceSynchronize());
+                CK(cudaStreamSynchronize(0));  // not the device: another thread may be recording a stream of it
                 ctx->dfree(tmp, tmp_words);
             } else {
                 pack_diags(f.get(), 0, n_diag, host, st);

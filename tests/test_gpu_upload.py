@@ -101,3 +101,54 @@ def test_device_upload_from_other_memory(where):
         g.device_status()
     finally:
         g.close()
+
+
+def test_uploads_beside_a_recording():
+    """While one thread records a stream, another uploads to a context of its own from the host."""
+    import threading
+
+    import torch
+
+    from paper_2605_17222_gb300 import binding, synth
+    ps = synth.param_set("toy")
+    g, other = binding.Context.from_params(ps), binding.Context.from_params(ps)
+    f = diagonals(ps, 4)
+    try:
+        fh = g.upload_diagonals(f)
+        want = lt_of(g, ps, fh)
+        ct = g.ct_from_host(np.stack([synth.uniform_mod(7 + c, "ct", ps.q, ps.n) for c in range(2)]))
+        out, stream = g.ct_empty(ps.L - 1), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        recording, uploaded, got = threading.Event(), threading.Event(), []
+
+        def record():
+            try:
+                g.graph_begin(stream)
+                g.lt_eval(ct, fh, "th", (1, 2, 2), out=out, stream=stream)
+                recording.set()
+                uploaded.wait(60)
+                got.append(g.graph_end(stream, keep=(ct, fh, out)))
+            except Exception as e:
+                got.append(e)
+                recording.set()
+
+        t = threading.Thread(target=record)
+        t.start()
+        recording.wait(60)
+        try:
+            theirs = other.upload_diagonals(f)
+            other.upload_rotation_key(1, np.broadcast_to(synth.uniform_mod(1, "k", ps.moduli, ps.n),
+                                                         (g.beta_max, 2, len(ps.moduli), ps.n)))
+        finally:
+            uploaded.set()
+            t.join()
+        assert not isinstance(got[0], Exception), got[0]
+        got[0].launch(stream)
+        torch.cuda.synchronize()
+        assert np.array_equal(out.numpy(), want)
+        assert np.array_equal(lt_of(other, ps, theirs), want)
+        got[0].close()
+        g.device_status()
+    finally:
+        g.close()
+        other.close()
