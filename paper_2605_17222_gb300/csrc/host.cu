@@ -1516,9 +1516,14 @@ static void put_diags(ckks_ctx* ctx, ckks_diags** out, uint32_t n_diag, int32_t 
         try {
             if (kind == cudaMemcpyHostToDevice) {
                 const size_t per = (size_t)(level + ctx->K) * ctx->N;
-                const u32 chunk = stage_diags(f.get(), n_diag);
-                tmp_words = per * chunk;
-                tmp = ctx->dalloc(tmp_words);
+                u32 chunk = stage_diags(f.get(), n_diag);
+                while (!tmp) try {  // less at a time where the device has no room for it
+                    tmp = ctx->dalloc(per * chunk);
+                    tmp_words = per * chunk;
+                } catch (const Fail& e) {
+                    if (e.st != CKKS_ENOMEM || chunk == 1) throw;
+                    chunk = (chunk + 1) / 2;
+                }
                 for (u32 d0 = 0; d0 < n_diag; d0 += chunk) {
                     const u32 n = std::min(chunk, n_diag - d0);
                     CK(cudaMemcpy(tmp, host + per * d0, per * n * 8, kind));

@@ -152,3 +152,27 @@ def test_uploads_beside_a_recording():
     finally:
         g.close()
         other.close()
+
+
+def test_host_upload_of_diagonals_in_little_memory():
+    """128 diagonals at N = 2^14 are 118 MB as stored and 168 MB on their way there: with room for half of
+    those, they are staged in smaller parts."""
+    from paper_2605_17222_gb300 import binding, synth
+    ps = synth.param_set("n14")
+    g = binding.Context.from_params(ps)
+    f, split = diagonals(ps, 128), (4, 8, 4)
+    key = np.ascontiguousarray(np.broadcast_to(synth.uniform_mod(1, "k", ps.moduli, ps.n),
+                                               (g.beta_max, 2, len(ps.moduli), ps.n)))
+    ct = np.stack([synth.uniform_mod(7 + c, "ct", ps.q, ps.n) for c in range(2)])
+    try:
+        with left((118 + 80) * MB):
+            staged = g.upload_diagonals(f)
+        for r in g.required_rotations("th", split, 128):
+            g.upload_rotation_key(r, key)
+        whole = g.upload_diagonals_device(binding.to_device(f))
+        ct = g.ct_from_host(ct)
+        got, want = (g.lt_eval(ct, x, "th", split)[0].numpy() for x in (staged, whole))
+        assert np.array_equal(got, want)
+        g.device_status()
+    finally:
+        g.close()
