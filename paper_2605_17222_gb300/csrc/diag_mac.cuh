@@ -491,9 +491,14 @@ bool try_ws(const DiagMacArgs& a, bool join, cudaStream_t st) {
     const u32 beta = BETA == WS_ANY ? a.beta : BETA;
     const u32 N = 1u << a.log_n;
     // one CTA's share, less the 1 KB that the system takes per CTA and the static
-    // barriers; past eight digits a CTA may need all of it for two stages
+    // barriers: of MINB CTAs, or of fewer where two stages need it, for a long j
+    // table or a key block with the high bytes of many more digits.  Eight digits,
+    // wide, (1,400,2) at N = 2^12 with three CTAs: 358 us, 887 by the plain kernel;
+    // packed, of 36, (1,16,4) at 2^14: 74 and 95; of 128, (1,8,4) at 2^12 with two:
+    // 23.2 and 25.3.  One CTA is slower than the plain kernel (of 160: 28.5 and
+    // 25.0), but past eight digits, whose every stage is large, it is not (see WS_ANY)
     const u32 tab = (4 * a.n2 + 15) & ~15u;
-    constexpr int MIN_CTAS = BETA == WS_ANY ? 1 : MINB;
+    constexpr int MIN_CTAS = BETA == WS_ANY ? 1 : 2;
     u32 ring = 0;
     for (int ctas = MINB; ctas >= MIN_CTAS; ctas--) {
         const u32 share = SM_SMEM / ctas - 1024 - 256;

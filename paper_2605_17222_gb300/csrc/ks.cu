@@ -218,8 +218,10 @@ __global__ void __launch_bounds__(BLK) k_ks_any(const __grid_constant__ KsArgs a
 // n1*n2 rotated ciphertexts to HBM.  DH-BSGS is the case n2 = 1, the diagonal
 // method n1 = 1, BSGS n2 = 1 over Q only.
 //
-// This plain form reads its operands straight from global memory; it runs the
-// shapes whose stages do not fit the staged kernel (about forty digits) and unaligned operands.
+// This plain form reads its operands straight from global memory; it runs what
+// the staged kernel does not take: stages that do not fit (about forty digits,
+// or up to eight of a key with well over a hundred), operands at an odd word,
+// and bases of more than DM_MAX_LIMBS limbs.
 template <int K3>
 __global__ void __launch_bounds__(THREADS, 2) k_diag_mac(const __grid_constant__ DiagMacArgs a, u32 l0) {
     const u32 N = 1u << a.log_n;
