@@ -36,15 +36,16 @@ class Request:
 
 
 def scratch_bytes(ctx, level: int, split) -> int:
-    """Device scratch one TH-BSGS LT takes at `level` with `split`: digit sets of
-    the inner and outer layers, the baby pairs, the giant-step accumulators and
-    the transform buffers (upper estimate)."""
+    """Device scratch one TH-BSGS LT takes at most at `level` with `split`, alone
+    or as one of a batch: digit sets with A_i beside them and B_i per baby index,
+    digits and accumulators per outer index (with a base offset every one is
+    rotated and there are two more accumulators), the transforms' sources and
+    the polynomials between a ModDown and its Decompose."""
     n1, n2, n3 = split
     ext = level + ctx.k
     beta = ctx.beta(level)
-    limbs = (n1 + max(n3 - 1, 0)) * beta * ext      # digit sets
-    limbs += 2 * n1 * ext + 2 * n3 * ext            # pairs and accumulators
-    limbs += (max(n1 - 1, n3 - 1, 1) + 2) * level   # moduli-switch buffers
+    limbs = (n1 + n3) * (beta + 2) * ext + 2 * ext
+    limbs += max(n1 - 1, n3) * (ext + level) + ctx.k + 2
     return limbs * 8 * ctx.N
 
 

@@ -85,3 +85,42 @@ def test_bsgs_in_little_memory():
         torch.cuda.empty_cache()
         pool.cu.cuMemPoolTrimTo(pool.pool, ctypes.c_size_t(0))
         g.close()
+
+
+@pytest.mark.parametrize("params,level,split,offset0", [
+    ("n14", 8, (1, 16, 4), 0), ("n14", 8, (1, 16, 4), 5), ("n14", 3, (4, 1, 16), 1), ("n14", 8, (16, 2, 2), 0),
+    ("setA", 2, (8, 1, 8), 0), ("setA", 5, (1, 1, 16), 3), ("n16", 24, (1, 16, 4), 1),
+])
+def test_serving_estimate_is_an_upper_one(params, level, split, offset0):
+    """The serving loop's scratch_bytes covers what an LT, and each of a batch, takes from the pool."""
+    import torch
+
+    from paper_2605_17222_gb300 import binding, synth
+    from paper_2605_17222_gb300.serving import scratch_bytes
+    ps = synth.param_set(params)
+    g, D = binding.Context.from_params(ps), int(np.prod(split))
+    pool = _DefaultPool(torch.cuda.current_device())
+    if not pool.cu:
+        pytest.skip("no driver library")
+    try:
+        key = synth.uniform_mod_device(1, "k", ps.moduli, ps.n, 2 * g.beta_max)
+        for r in g.required_rotations("th", split, D, offset0=offset0):
+            g.upload_rotation_key_device(r, key)
+        f = g.diags_create(D, offset0=offset0)
+        g.diags_write(f, 0, synth.uniform_mod_device(2, "f", ps.moduli, ps.n, D))
+        cts = [g.ct_wrap(synth.uniform_mod_device(3 + i, "c", ps.q[:level], ps.n, 2), level) for i in range(3)]
+        outs = [g.ct_empty(level - 1) for _ in cts]
+        one = scratch_bytes(g, level, split)
+        for count, run in ((1, lambda: g.lt_eval(cts[0], f, "th", split, out=outs[0])),
+                           (3, lambda: g.lt_eval_batch(cts, [f] * 3, ["th"] * 3, [split] * 3, outs))):
+            run()
+            torch.cuda.synchronize()
+            pool.reset_high()
+            used = pool.get(CU_MEMPOOL_ATTR_USED_MEM_CURRENT)
+            run()
+            torch.cuda.synchronize()
+            peak = pool.get(CU_MEMPOOL_ATTR_USED_MEM_HIGH) - used
+            assert peak <= count * one, f"{count} LTs: {peak / MB:.1f} MB, estimated {count * one / MB:.1f}"
+        g.device_status()
+    finally:
+        g.close()
