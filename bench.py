@@ -549,8 +549,7 @@ def run_ours(args, dist: Dist):
                                f"dnum 6, {D} consecutive diagonals, one ciphertext at the top level",
                    "algo": algo, "split": list(split3), "parallelism": f"replicas x{dist.world}",
                    **({"dh_schedule": dh_sched} if dh_sched else {}),
-                   **({"k6_tile": {"outer_per_cta": tile[0] or "default", "positions_per_cta": tile[1] or "default"}}
-                      if tile else {}),
+                   **({"k6_tile": {"outer_per_cta": tile[0] or "default"}} if tile else {}),
                    "split_choice": ("given" if args.split else "the diagonal method has one split" if tuned_ms is None
                                     else f"autotuned over the cost model's best candidates ({tuned_ms:.3f} ms "
                                          f"when measured)"),
@@ -878,7 +877,7 @@ def run_paper_shape(args, dist: Dist):
         "config": {"workload": f"dense LT with the paper's {cfg['params']}: N=2^{ps.log_n}, L+1={ps.L}, "
                                f"alpha={ps.alpha}, beta={g.beta(lvl)}, n={Dn}, split {split}",
                    "split": list(split), "autotuned": {"split": list(tuned_split), "ms": round(tuned_ms, 4),
-                                                        "k6_tile": list(tile) if tile else None}},
+                                                        "k6_tile": {"outer_per_cta": tile[0] or "default"} if tile else None}},
         "paper_fpga_ms_context": cfg["fpga_ms"],
         "paper_fpga_offchip": fpga_offchip(cfg["params"]),
         "hbm_roofline_lt": {"compulsory_bytes": comp, "frac": round(comp / (ms / 1e3) / 1e9 / peak, 4)},

@@ -248,11 +248,16 @@ int32_t lt_candidate_splits(const ckks_ctx* ctx, lt_algo algo, uint32_t level, u
                             uint32_t cap);
 
 /* The cost model that ranks the splits (the key-memory / compute trade-off
- * of Sec. III) for one LT: hbm_bytes = the DRAM bytes it counts (diagonals,
- * distinct keys, input and output, and each Decompose's digits written and
- * read once; -1 for BSGS, whose model counts them differently) and seconds =
- * its time estimate (bytes over a fitted bandwidth plus the NTT butterflies
- * and the multiply-accumulates over fitted kernel rates).  DH-BSGS is
+ * of Sec. III) for one LT: hbm_bytes = the bytes it counts, every word at 8
+ * (diagonals, distinct keys, input and output, and each Decompose's digits
+ * written and read once; -1 for BSGS, whose model counts them differently), and
+ * seconds = its time estimate (bytes over a fitted bandwidth plus the NTT
+ * butterflies and the multiply-accumulates over fitted kernel rates).  They are
+ * there to compare splits by: the rates are kept as they were first fitted, so
+ * that a call without a split keeps its split, and moduli between 2^32 and 2^40
+ * are stored at 5 bytes a word, so an LT reads fewer bytes and takes less time
+ * (N = 2^16, level 24, 256 diagonals, (1,64,4): 17.2 GB and 3.45 ms by the
+ * model, 12.6 GB and 2.65 ms measured).  DH-BSGS is
  * modelled in the schedule the model prefers (see lt_dh_schedule).  EINVAL
  * on a bad level or split. */
 ckks_status lt_model_estimate(const ckks_ctx* ctx, lt_algo algo, uint32_t level, uint32_t n_diag,

@@ -366,7 +366,8 @@ class Context:
         return "fused" if r == 1 else "baby"
 
     def model_estimate(self, algo: str, level: int, n_diag: int, split):
-        """(DRAM bytes, seconds) the split-selection cost model assigns to one LT (lt_model_estimate)."""
+        """(bytes at 8 a word, seconds) the split-selection cost model assigns to one LT, to compare
+        splits by (lt_model_estimate)."""
         sp = Split(*(tuple(split) + (1,) * (3 - len(split))))
         b, t = ctypes.c_double(), ctypes.c_double()
         check(lib().lt_model_estimate(self.h, ALGOS[algo], level, n_diag, ctypes.byref(sp), ctypes.byref(b),

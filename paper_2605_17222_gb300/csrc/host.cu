@@ -491,13 +491,14 @@ void op_moddown_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& xs,
 // NTT words for the digits' own limbs, as the ModDown tail of forward jobs that
 // join the conversions' launch and write the digits in place.  Five launches
 // and no ModDown polynomial in memory, where the two steps one after the other
-// are eight and write it, read it back and copy it (N = 2^16 level 9, (2,8,4):
-// 688 -> 670 us).  The price is the special limbs' conversion a second time,
-// K products a word, so it pays where launches count: up to 3 * 2^20 words of
-// Q limbs (N = 2^16 level 24, three polynomials, 4.5 * 2^20: 2.818 ms fused, 2.810
-// not; N = 2^15 level 11, 2.3 * 2^20: 574 and 577 us), or 2^20 with more than
-// four special limbs (Set-B, K = 8, 2^21.6: 1.45 and 1.435 ms; Set-A, K = 5,
-// 2^19.2: 1.367 and 1.381 ms).
+// are eight and write it, read it back and copy it.  The price is the special
+// limbs' conversion a second time, K products a word, so it pays where launches
+// count.  Both forms over 22 LTs of six parameter sets, gain of the merged one by
+// words of Q limbs in units of 2^20: up to four special limbs 0.05 (toy) 22%,
+// 0.4 to 0.9 3 to 8%, 1.5 to 1.9 1 to 4%, 2.9 to 3.0 0.2 to 1.5%, 3.9 to 5.5 -1.1 to
+// -0.4%, hence the line at 3; with five (Set-A) 0.3 13%, 0.6 7%, 1.05 2%, with
+// eight (Set-B) 0.4 to 0.5 5%, 1.5 0.8%, 3.5 -1.2%: the line at 1 gives away less
+// than 1%.
 // Y: scratch [count][K + level][N].
 void op_moddown_decompose_batch(ckks_ctx* C, u32 level, const std::vector<const u64*>& xs,
                                 const std::vector<u64*>& digits, u32 slots, u64* Y, cudaStream_t st) {
@@ -1069,10 +1070,10 @@ std::vector<int64_t> rotations(const ckks_ctx* C, lt_algo algo, const lt_split& 
 }  // namespace
 
 // ------------------------------------------------------------------ split choice (autotuner model)
-// Time model of one LT on this GPU, phase by phase: the diagonal kernel K6 at
-// the slower of its DRAM bytes and its multiply-accumulates, the key-switch
-// inner products at their DRAM bytes, and the Decompose / ModDown transforms
-// at their NTT butterflies.  The split with the smallest estimate wins.
+// Time model of one LT, phase by phase: the diagonal kernel K6 at the slower of
+// its bytes and its multiply-accumulates, the key-switch inner products at
+// their bytes, and the Decompose / ModDown transforms at their NTT butterflies.
+// The split with the smallest estimate wins.
 namespace {
 // The model over a TH-shaped schedule (n1, n2, n3) = (n'1, n'2, n'3): with
 // n2 = 1 there is no middle layer, so neither the baby steps' ModDown and
@@ -1081,16 +1082,18 @@ namespace {
 struct ModelEst {
     double bytes, ntt_s, mac_s, seconds;
 };
-// Rates of this library's kernels on GB300, fitted to LTs measured at N = 2^16,
-// level 24, D = 256 over the splits (1,64,4), (2,32,4), (4,16,4), (2,16,8),
-// (1,32,8) (time within 3% of each; DRAM bytes within 2% of ncu's per-LT sum
-// for (1,64,4), (2,32,4) and (4,8,8)):
+// The ranking decides which split, and so which residues, a call without a split
+// gives; it therefore stays as it was fitted, on an earlier build that stored
+// every word of a key or diagonal at 8 bytes and ran at
 //   effective HBM bandwidth of the streaming kernels                6.2e12 B/s
 //   K6 multiply-accumulates, 4 or fewer outer indices per CTA       9.5e11 /s
 //                            8 outer indices per CTA                7.0e11 /s
-//   NTT butterflies (about 1.35 us per 2^16-point limb transform)   3.9e11 /s
-//   DRAM traffic of a limb transform: 2.75 limbs (input, the two passes'
+//   NTT butterflies                                                 5.8e11 /s
+//   a limb transform's traffic: 2.75 limbs (input, the two passes'
 //   intermediate mostly through DRAM, output)
+// (fitted at N = 2^16, level 24, D = 256 over six splits).  What it gives is a
+// figure to compare splits by, not this build's bytes or time: (1,64,4) there is
+// 17.2 GB and 3.45 ms to the model, 12.6 GB (5-byte words) and 2.65 ms measured.
 constexpr double M_BW = 6.2e12, M_MAC4 = 9.5e11, M_MAC8 = 7.0e11, M_NTT = 5.8e11, M_FIXED = 1e-4;
 constexpr double M_NTT_LIMBS = 2.75;
 

@@ -15,8 +15,12 @@ namespace ckks {
 // tables overlap the end of the kernel before it, and pdl_wait() holds it
 // before it touches memory that an earlier kernel wrote (or that it
 // overwrites).  pdl_wait() returns when the kernel before it is complete and
-// its writes are visible; every kernel of an evaluation calls it, so all
-// earlier ones are complete too.  Who launches early was measured kernel by
+// its writes are visible; every CTA of an evaluation's kernels calls it, so all
+// earlier ones are complete too.  The exception is the packed diagonal kernel
+// behind a wide one: it starts early, and only its last CTA waits, at its end
+// (diag_mac.cuh).  That is sound because the wide launch is never early (what
+// both read was complete when it started) and that CTA keeps the packed grid
+// from completing before the wide one.  Who launches early was measured kernel by
 // kernel: the second pass of each transform and the gathers always (N = 2^14
 // BSGS 1.92 -> 1.70 ms, N = 2^16 level 9 708 -> 689 us); the inverse row pass
 // in small grids (1.70 -> 1.61); the forward column pass, the key products and

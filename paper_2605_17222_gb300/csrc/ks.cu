@@ -12,7 +12,7 @@
 // warp's gathered load touches exactly the same 256 bytes as a plain load.
 //
 // Sums of products stay in carry-free accumulators of split operands (Sum40,
-// Sum60, Outer3) and are reduced once (PE modes CWPM-ACC / CM-ACC of Sec. V,
+// Sum60, WsAcc) and are reduced once (PE modes CWPM-ACC / CM-ACC of Sec. V,
 // done lazily).
 #include "kernels.h"
 #include "ks_products.cuh"

@@ -233,11 +233,6 @@ __device__ __forceinline__ u64 canon8(u64 x, u64 q) {
     return x >= q ? x - q : x;
 }
 
-__device__ __forceinline__ u64 mul_mod(u64 a, u64 b, const ModC& m) {
-    U128 p{a * b, __umul64hi(a, b)};
-    return reduce128(p, m);
-}
-
 // Source index of the NTT-domain automorphism x -> x^g in bit-reversed
 // storage (Eq. 7): output word s reads word brv(((g (2 brv(s) + 1)) mod 2N - 1) / 2).
 // 2N divides 2^32, so the product may wrap.
