@@ -153,12 +153,17 @@ struct WsCtx {
 // (BETA is exact, outer indices past k_count compute on stale words that are
 // never stored), so that the middle layer's shared-memory loads are issued
 // together.  The diagonal words are read after its products, whose registers
-// they then take ((1,64,4) 1.78 -> 1.74 ms, Set-B 0.62 -> 0.58), but for the wide
-// limbs with one digit, which have registers to spare (Set-A 0.92, 0.96 late).
+// they then take ((1,64,4) 1.78 -> 1.74 ms, Set-B 0.62 -> 0.58), but for wide limbs
+// with one digit and eight outer indices, where two CTAs per SM leave registers
+// for both: Set-A (16,16,16) 0.920 ms early, 0.963 late; (4,16,8) 146 us, 152; Set-B
+// at level 8, (1,32,8) 372, 387.  With four they are even (88 and 88 us, 221 and
+// 221), with one or two early is the slower (Set-A (4,16,2) 70 us, 68 late;
+// (1,64,1) 67, 66; Set-B (1,32,2) 166, 160; (1,32,1) 147, 143).
 template <int K3, int BETA, int CLS>
 __device__ __forceinline__ void ws_compute(const WsCtx& c) {
     constexpr u32 FULLM = 0xffffffffu;
     constexpr u32 FB = CLS == C40 ? BLK * 5 : BLK * 8;  // diagonal block
+    constexpr bool EARLY_F = BETA == 1 && K3 >= 8;      // wide limbs: diagonal words before the products (above)
     const DiagMacArgs& a = c.a;
     const u32 l = c.l, n1 = a.n1, n1n2 = a.n1 * a.n2;
     const ModC m = c.m;
@@ -276,7 +281,7 @@ __device__ __forceinline__ void ws_compute(const WsCtx& c) {
                 ulonglong2 k[BETA];
 #pragma unroll
                 for (int b = 0; b < BETA; b++) k[b] = kp[b * BLK];
-                if constexpr (BETA == 1) {
+                if constexpr (EARLY_F) {
                     load_f(st);
                     release();
                 }
@@ -290,7 +295,7 @@ __device__ __forceinline__ void ws_compute(const WsCtx& c) {
                     split30(k[b].y, kl, kh);
                     s1.mac(dl, dh, kl, kh);
                 }
-                if constexpr (BETA > 1) {
+                if constexpr (!EARLY_F) {
                     load_f(st);
                     release();
                 }
