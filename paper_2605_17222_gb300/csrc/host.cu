@@ -903,6 +903,9 @@ void sched_th_batch(ckks_ctx* C, u32 level, const std::vector<LtIO>& ios, const 
 // at most BSGS_SCRATCH bytes (one rotation at least), and where the device has
 // not even that left, the chunks are halved until they fit: one rotation at a
 // time takes no more than a sequence of ckks_ks_inner and ckks_moddown does.
+// The sums by chunk read and write the accumulators once a chunk: at N = 2^16
+// level 23, 26 giant steps in chunks of four, 6.92 ms against 6.88 for one sum
+// over all outputs, which took 0.6 GB more.
 constexpr size_t BSGS_SCRATCH = size_t(512) << 20;
 
 void sched_bsgs(ckks_ctx* C, u32 level, LtIO io, const ckks_diags* f, u32 n1, u32 n2, cudaStream_t st, u32 tile = 0) {
